@@ -70,6 +70,7 @@ static void free_plan(dd_plan *p)
     if (p->d_gen) cudaFree(p->d_gen);
     if (p->d_partials) cudaFree(p->d_partials);
     if (p->d_params) cudaFree(p->d_params);
+    if (p->d_fin) cudaFree(p->d_fin);
     if (p->d_wsorted) cudaFree(p->d_wsorted);
     if (p->d_cands) cudaFree(p->d_cands);
     if (p->d_count) cudaFree(p->d_count);
@@ -241,6 +242,8 @@ int plan_create(int32_t nchans, double fch1_mhz, double foff_mhz, double tsamp_s
         e = cudaMalloc(&p->d_wsorted, ws.size() * sizeof(int32_t));
         if (e == cudaSuccess) e = cudaMemcpy(p->d_wsorted, ws.data(), ws.size() * 4, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMalloc(&p->d_params, sizeof(SearchParams));
+        if (e == cudaSuccess) e = cudaMalloc(&p->d_fin, sizeof(FinScratch));
+        if (e == cudaSuccess) e = cudaMemset(&p->d_fin->ticket, 0, sizeof(unsigned int));
         if (e == cudaSuccess) e = cudaMalloc(&p->d_count, sizeof(unsigned long long));
         if (e == cudaSuccess) e = cudaMallocHost(&p->h_count, sizeof(unsigned long long));
         if (e == cudaSuccess) e = cudaMallocHost(&p->h_params, sizeof(SearchParams));

@@ -27,6 +27,15 @@ struct SearchParams {
     long long thr_i[64];         // floor(T_w) (integer compare is then exact)
 };
 
+// Scratch of the statistics finalisation: each block's merged record, and how
+// many blocks have finished (0 between launches).
+struct FinI { long long n, sum; unsigned long long q_lo, q_hi; };
+constexpr int kFinBlocks = 512;
+struct FinScratch {
+    union { StatF f[kFinBlocks]; FinI i[kFinBlocks]; };
+    unsigned int ticket;
+};
+
 constexpr int kMaxWidths = 64;
 
 // Per-DM-row statistics and thresholds (search option: statistics of each DM
@@ -77,6 +86,7 @@ struct dd_plan {
     const void *stats_out = nullptr;       // out buffer the partials describe
     // search
     dd::SearchParams *d_params = nullptr;
+    dd::FinScratch *d_fin = nullptr;
     int32_t *d_wsorted = nullptr;          // widths sorted ascending: [nw] widths, [nw] indices
     dd_candidate *d_cands = nullptr;
     int64_t cand_cap = 0;

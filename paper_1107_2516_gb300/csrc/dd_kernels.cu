@@ -188,85 +188,123 @@ stats_kernel(const void *__restrict__ out_, int64_t total, void *__restrict__ pa
 // in double (Section 3's n-sigma test applied to boxcar sums).  Each
 // threshold is stored as the largest float <= T_w and as floor(T_w), so the
 // kernels' FP32 / integer comparisons decide B_w > T_w exactly as a double
-// comparison of the same B_w would.  One block of 1024 threads.
+// comparison of the same B_w would.  It also clears the hit count that the
+// search adds to.
+//
+// The LOFAR-like plan leaves 64 288 partials (1.5 MB).  One block of 1024
+// threads took 122 us for them: two passes of dependent loads by one SM, and
+// FP64 at two lanes a clock.  Here each block merges its own run of about
+// kFinRun partials and the last block to finish (a ticket in the plan's
+// scratch) merges the blocks' records with the same code, so the loads and
+// the FP64 work spread over the SMs: 122 -> 10 us there, 291 -> 16 us for
+// the 168 756 partials of the subband plan.  The runs depend on the number
+// of partials alone: the result is the same from call to call.
 // ---------------------------------------------------------------------------
-constexpr int kFinThreads = 1024;
+constexpr int kFinThreads = 128;
+constexpr int kFinRun = 512;        // partials per block (at least; kFinBlocks blocks at most)
+static_assert(kFinThreads >= kMaxWidths, "one thread per width forms the thresholds");
+
+template <typename T>
+__device__ __forceinline__ T fin_block_sum(T v, T *sh)
+{
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    T r = sh[0];
+#pragma unroll
+    for (int w = 1; w < kFinThreads / 32; ++w) r += sh[w];
+    return r;
+}
+
+// Records [lo, hi) merged, in every thread of the block: two passes, no
+// division per record, mean = sum n_b*mean_b / N, M2 = sum [M2_b + n_b*(mean_b - mean)^2].
+__device__ __forceinline__ StatF fin_merge(const StatF *p, int64_t lo, int64_t hi)
+{
+    __shared__ double sh[kFinThreads / 32];
+    double n = 0, s = 0, q = 0;
+    for (int64_t i = lo + threadIdx.x; i < hi; i += kFinThreads) { n += p[i].n; s += p[i].n * p[i].mean; }
+    StatF r;
+    r.n = fin_block_sum(n, sh);
+    s = fin_block_sum(s, sh);
+    r.mean = r.n > 0 ? s / r.n : 0.0;
+    for (int64_t i = lo + threadIdx.x; i < hi; i += kFinThreads) {
+        const double e = p[i].mean - r.mean;
+        q += p[i].m2 + p[i].n * e * e;
+    }
+    r.m2 = fin_block_sum(q, sh);
+    return r;
+}
+
+// The same for integer records: exact sums, the squares in 128 bits.
+__device__ __forceinline__ FinI fin_merge(const StatI *p, const FinI *f, int64_t lo, int64_t hi)
+{
+    __shared__ long long sh[kFinThreads / 32];
+    __shared__ unsigned long long shu[kFinThreads / 32];
+    long long n = 0, s = 0;
+    unsigned long long q0 = 0, q1 = 0, q2 = 0;   // 32-bit limbs: sums of up to 2^32 records stay exact
+    for (int64_t i = lo + threadIdx.x; i < hi; i += kFinThreads) {
+        const unsigned long long l = p ? p[i].sumsq : f[i].q_lo, h = p ? 0ull : f[i].q_hi;
+        n += p ? p[i].n : f[i].n;
+        s += p ? p[i].sum : f[i].sum;
+        q0 += l & 0xffffffffull; q1 += l >> 32; q2 += h;
+    }
+    FinI r;
+    r.n = fin_block_sum(n, sh);
+    r.sum = fin_block_sum(s, sh);
+    q0 = fin_block_sum(q0, shu);
+    q1 = fin_block_sum(q1, shu);
+    q2 = fin_block_sum(q2, shu);
+    const unsigned __int128 q = (unsigned __int128)q0 + ((unsigned __int128)q1 << 32) + ((unsigned __int128)q2 << 64);
+    r.q_lo = (unsigned long long)q;
+    r.q_hi = (unsigned long long)(q >> 64);
+    return r;
+}
 
 template <bool kInt>
 __global__ void __launch_bounds__(kFinThreads)
 finalize_kernel(const void *__restrict__ partials, int64_t np, const int32_t *__restrict__ widths,
-                int nw, double k, SearchParams *__restrict__ prm)
+                int nw, double k, SearchParams *__restrict__ prm, unsigned long long *__restrict__ count,
+                FinScratch *__restrict__ scr)
 {
-    __shared__ double mu_s, sg_s;
-    if constexpr (kInt) {
-        __shared__ long long sn[kFinThreads], ss[kFinThreads];
-        __shared__ unsigned long long sq_lo[kFinThreads], sq_hi[kFinThreads];
-        const StatI *p = reinterpret_cast<const StatI *>(partials);
-        long long n = 0, s = 0;
-        unsigned __int128 q = 0;
-        for (int64_t i = threadIdx.x; i < np; i += kFinThreads) {
-            n += p[i].n; s += p[i].sum; q += (unsigned __int128)p[i].sumsq;
-        }
-        sn[threadIdx.x] = n; ss[threadIdx.x] = s;
-        sq_lo[threadIdx.x] = (unsigned long long)q;
-        sq_hi[threadIdx.x] = (unsigned long long)(q >> 64);
-        __syncthreads();
-        for (int h = kFinThreads / 2; h > 0; h >>= 1) {
-            if (threadIdx.x < h) {
-                const int o = threadIdx.x + h;
-                sn[threadIdx.x] += sn[o];
-                ss[threadIdx.x] += ss[o];
-                unsigned __int128 a = ((unsigned __int128)sq_hi[threadIdx.x] << 64) | sq_lo[threadIdx.x];
-                unsigned __int128 b = ((unsigned __int128)sq_hi[o] << 64) | sq_lo[o];
-                a += b;
-                sq_lo[threadIdx.x] = (unsigned long long)a;
-                sq_hi[threadIdx.x] = (unsigned long long)(a >> 64);
-            }
-            __syncthreads();
-        }
+    using Rec = typename std::conditional<kInt, FinI, StatF>::type;
+    __shared__ bool last_s;
+    const int64_t lo = np * blockIdx.x / gridDim.x, hi = np * (blockIdx.x + 1) / gridDim.x;
+    Rec r;
+    if constexpr (kInt) r = fin_merge(static_cast<const StatI *>(partials), nullptr, lo, hi);
+    else r = fin_merge(static_cast<const StatF *>(partials), lo, hi);
+    if (gridDim.x > 1) {
+        Rec *rec;
+        if constexpr (kInt) rec = scr->i; else rec = scr->f;
         if (threadIdx.x == 0) {
-            const long long N = sn[0], S = ss[0];
-            const unsigned __int128 Q = ((unsigned __int128)sq_hi[0] << 64) | sq_lo[0];
-            // N*Q - S^2 >= 0 exactly (Cauchy-Schwarz), then one rounding each.
-            const __int128 num = (__int128)((unsigned __int128)N * Q) - (__int128)S * (__int128)S;
-            const double dn = (double)N;
-            mu_s = (double)S / dn;
-            sg_s = sqrt((double)num / (dn * dn));
+            rec[blockIdx.x] = r;
+            __threadfence();
+            last_s = atomicAdd(&scr->ticket, 1u) == gridDim.x - 1;
         }
-    } else {
-        // Two passes over the partials, no division per partial:
-        //   mean = sum n_b*mean_b / N,  M2 = sum [M2_b + n_b*(mean_b - mean)^2].
-        __shared__ double sa[kFinThreads], sb[kFinThreads];
-        const StatF *p = reinterpret_cast<const StatF *>(partials);
-        double n = 0, s = 0;
-        for (int64_t i = threadIdx.x; i < np; i += kFinThreads) { n += p[i].n; s += p[i].n * p[i].mean; }
-        sa[threadIdx.x] = n; sb[threadIdx.x] = s;
         __syncthreads();
-        for (int h = kFinThreads / 2; h > 0; h >>= 1) {
-            if (threadIdx.x < h) { sa[threadIdx.x] += sa[threadIdx.x + h]; sb[threadIdx.x] += sb[threadIdx.x + h]; }
-            __syncthreads();
-        }
-        const double N = sa[0];
-        const double M = N > 0 ? sb[0] / N : 0.0;
-        __syncthreads();
-        double q = 0;
-        for (int64_t i = threadIdx.x; i < np; i += kFinThreads) {
-            const double e = p[i].mean - M;
-            q += p[i].m2 + p[i].n * e * e;
-        }
-        sa[threadIdx.x] = q;
-        __syncthreads();
-        for (int h = kFinThreads / 2; h > 0; h >>= 1) {
-            if (threadIdx.x < h) sa[threadIdx.x] += sa[threadIdx.x + h];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) { mu_s = M; sg_s = sqrt(sa[0] / N); }
+        if (!last_s) return;
+        __threadfence();
+        if constexpr (kInt) r = fin_merge(nullptr, rec, 0, gridDim.x);
+        else r = fin_merge(rec, 0, gridDim.x);
+        if (threadIdx.x == 0) scr->ticket = 0;      // for the next launch
     }
-    __syncthreads();
-    if (threadIdx.x == 0) { prm->mu = mu_s; prm->sigma = sg_s; prm->nw = nw; }
+    double mu, sg;
+    if constexpr (kInt) {
+        const unsigned __int128 Q = ((unsigned __int128)r.q_hi << 64) | r.q_lo;
+        // N*Q - S^2 >= 0 exactly (Cauchy-Schwarz), then one rounding each.
+        const __int128 num = (__int128)((unsigned __int128)r.n * Q) - (__int128)r.sum * (__int128)r.sum;
+        const double dn = (double)r.n;
+        mu = (double)r.sum / dn;
+        sg = sqrt((double)num / (dn * dn));
+    } else {
+        mu = r.mean;
+        sg = sqrt(r.m2 / r.n);
+    }
+    if (threadIdx.x == 0) { prm->mu = mu; prm->sigma = sg; prm->nw = nw; *count = 0; }
     if (threadIdx.x < nw) {
         const double w = (double)widths[threadIdx.x];
-        const double T = w * mu_s + k * sg_s * sqrt(w);
+        const double T = w * mu + k * sg * sqrt(w);
         prm->thr_f[threadIdx.x] = __double2float_rd(T);
         double f = floor(T);
         f = fmin(fmax(f, -4.0e18), 4.0e18);
@@ -368,14 +406,11 @@ row_stats_kernel(const void *__restrict__ out_, int64_t nout, const int32_t *__r
 }
 
 // ---------------------------------------------------------------------------
-// Boxcar threshold search.  Block = one DM row x kSearchTile samples; thread
-// owns kSearchPer consecutive samples.  For the widths in ascending order it
-// extends B_w at its first sample from the previous width's sum, then slides
-// it along its samples (B_w(t+1) = B_w(t) + x[t+w] - x[t]), testing
-// B_w > T_w at each (t, w).  Only FP32 (or integer) arithmetic runs here;
-// hits are appended with one atomic each and their S/N is formed afterwards
-// by cand_snr_kernel.  The shared tile is padded one word per 16 so the
-// per-thread windows fall in distinct banks.
+// Boxcar threshold search.  Block = one DM row x kSearchTile samples.  Both
+// kernels test a whole run of samples per thread by its largest boxcar sum
+// (one max per sample and width, one comparison per run and width); only runs
+// whose largest sum is a hit are gone through again sample by sample.  A hit's
+// S/N, (B_w - w*mu) / (sigma*sqrt(w)) in double, is formed with its record.
 // ---------------------------------------------------------------------------
 constexpr int kSearchThreads = 256;
 constexpr int kSearchPer = 16;
@@ -383,6 +418,28 @@ constexpr int kSearchTile = kSearchThreads * kSearchPer;
 
 __host__ __device__ __forceinline__ int spad(int i) { return i + (i >> 4); }
 
+// S/N and record of one hit into slot pos.
+__device__ __forceinline__ void put_candidate(dd_candidate *cands, int64_t cap, unsigned long long pos, int row, int w,
+                                              int width_idx, int64_t t, double value, const SearchParams *prm,
+                                              const RowParams *rp)
+{
+    if ((int64_t)pos >= cap) return;
+    const double dw = (double)w;
+    const double mu = rp ? rp[row].mu : prm->mu, sg = rp ? rp[row].sigma : prm->sigma;
+    dd_candidate c;
+    c.dm_idx = row; c.width_idx = width_idx; c.t = t;
+    c.snr = (float)((value - dw * mu) / (sg * sqrt(dw)));
+    c.reserved = 0.f; c.value = value;
+    cands[pos] = c;
+}
+
+// Any widths: thread = kSearchPer consecutive samples.  For the widths in
+// ascending order it extends B_w at its first sample from the previous
+// width's sum, then slides it along its samples (B_w(t+1) = B_w(t) + x[t+w] -
+// x[t]); its own samples x[t] stay in registers.  The shared tile is padded
+// one word per 16, so that the threads' windows fall in distinct banks; the
+// step over a pad comes at the same sample for every thread (it depends on w
+// alone), so addresses cost no arithmetic per thread.
 template <bool kInt>
 __global__ void __launch_bounds__(kSearchThreads)
 search_kernel(const void *__restrict__ out_, int64_t nout,
@@ -394,155 +451,271 @@ search_kernel(const void *__restrict__ out_, int64_t nout,
     using Acc = typename std::conditional<kInt, long long, float>::type;
     extern __shared__ __align__(16) unsigned char sraw[];
     __shared__ int sw[kMaxWidths], sidx[kMaxWidths];
-    __shared__ float thf[kMaxWidths];
-    __shared__ long long thi[kMaxWidths];
+    __shared__ Acc sthr[kMaxWidths];
     T *x = reinterpret_cast<T *>(sraw);
     const int row = blockIdx.y;
     const int64_t t0 = (int64_t)blockIdx.x * kSearchTile;
     const int len = kSearchTile + wmax - 1;
     if (threadIdx.x < nw) {
+        const int o = wsorted[nw + threadIdx.x];
         sw[threadIdx.x] = wsorted[threadIdx.x];
-        sidx[threadIdx.x] = wsorted[nw + threadIdx.x];
-        thf[threadIdx.x] = rp ? rp[blockIdx.y].thr_f[sidx[threadIdx.x]] : prm->thr_f[sidx[threadIdx.x]];
-        thi[threadIdx.x] = rp ? rp[blockIdx.y].thr_i[sidx[threadIdx.x]] : prm->thr_i[sidx[threadIdx.x]];
+        sidx[threadIdx.x] = o;
+        if constexpr (kInt) sthr[threadIdx.x] = rp ? rp[row].thr_i[o] : prm->thr_i[o];
+        else sthr[threadIdx.x] = rp ? rp[row].thr_f[o] : prm->thr_f[o];
     }
-    const T *src = reinterpret_cast<const T *>(out_) + (size_t)row * nout;
-    for (int i = threadIdx.x; i < len; i += kSearchThreads) {
-        const int64_t t = t0 + i;
-        x[spad(i)] = t < nout ? src[t] : (T)0;
+    const T *src = reinterpret_cast<const T *>(out_) + (size_t)row * nout + t0;
+    const int64_t avail = nout - t0;
+    {
+        T r[kSearchPer];
+#pragma unroll
+        for (int q = 0; q < kSearchPer; ++q) {
+            const int i = q * kSearchThreads + threadIdx.x;
+            r[q] = i < avail ? __ldcs(src + i) : (T)0;
+        }
+#pragma unroll
+        for (int q = 0; q < kSearchPer; ++q) x[spad(q * kSearchThreads + threadIdx.x)] = r[q];
     }
+    for (int i = kSearchTile + threadIdx.x; i < len; i += kSearchThreads) x[spad(i)] = i < avail ? src[i] : (T)0;
     __syncthreads();
     const int base = threadIdx.x * kSearchPer;
-    const int64_t tb = t0 + base;
-    if (tb >= nout) return;
+    const T *xb = x + spad(base);                  // this thread's samples, then a pad after every 16
+    if (base >= avail) return;
+    T own[kSearchPer];
+#pragma unroll
+    for (int i = 0; i < kSearchPer; ++i) own[i] = xb[i];
     Acc b0 = 0;          // running B_w at the thread's first sample
     int wprev = 0;
     for (int p = 0; p < nw; ++p) {
         const int w = sw[p];
-        for (int j = wprev; j < w; ++j) b0 += (Acc)x[spad(base + j)];
+        for (int j = wprev; j < w; ++j) b0 += (Acc)xb[spad(j)];
         wprev = w;
-        Acc b = b0;
+        const Acc thr = sthr[p];
+        // x[base + w - 1 + i] for i >= 1: a step over the pad at i == pad
+        const T *xw = xb + spad(w - 1);
+        const int pad = kSearchPer - ((w - 1) & (kSearchPer - 1));
+        Acc b = b0, m = b0;
+#pragma unroll
+        for (int i = 1; i < kSearchPer; ++i) {
+            b += (Acc)xw[i + (i >= pad ? 1 : 0)] - (Acc)own[i - 1];
+            if constexpr (kInt) m = b > m ? b : m;
+            else m = fmaxf(m, b);
+        }
+        if (!(m > thr)) continue;
+        // a hit in this run: its samples one by one (the same sums again)
+        b = b0;
+#pragma unroll 1
         for (int i = 0; i < kSearchPer; ++i) {
-            const int64_t t = tb + i;
+            const int64_t t = t0 + base + i;
             if (t + w > nout) break;
-            if (i > 0) b += (Acc)x[spad(base + i - 1 + w)] - (Acc)x[spad(base + i - 1)];
-            bool hit;
-            if constexpr (kInt) hit = b > thi[p];
-            else hit = b > thf[p];
-            if (hit) {
-                const unsigned long long pos = atomicAdd(count, 1ull);
-                if ((int64_t)pos < cap) {
-                    dd_candidate c;
-                    c.dm_idx = row; c.width_idx = sidx[p]; c.t = t;
-                    c.snr = 0.f; c.reserved = 0.f; c.value = (double)b;
-                    cands[pos] = c;
-                }
-            }
+            if (i > 0) b += (Acc)xw[i + (i >= pad ? 1 : 0)] - (Acc)xb[i - 1];
+            if (b > thr) put_candidate(cands, cap, atomicAdd(count, 1ull), row, w, sidx[p], t, (double)b, prm, rp);
         }
     }
 }
 
-// The same search for the common width set {1, 2, 4, ..., 2^(K-1)}.  The
-// tile is staged with kSearchPer independent loads per thread; each thread
-// then copies its kSearchPer samples plus the 2^(K-1) - 1 that follow into
-// registers and forms the boxcars as a doubling tree, B_2w(i) = B_w(i) +
-// B_w(i + w): one add per sample and width, no shared-memory traffic in the
-// loop (the sliding form needs two shared words per sample and width).
-// Integer data stay in int32 (at most 65536 channels x 255 x 64 < 2^31).
+// The same search for the common width set {1, 2, 4, ..., 2^(K-1)}: each
+// thread takes kPow2Per consecutive samples and the 2^(K-1) - 1 that follow
+// into registers and forms the boxcars as a doubling tree, B_2w(i) = B_w(i) +
+// B_w(i + w): one add per sample and width, two at a time from w = 4 on
+// (add.f32x2).  Integer data stay in int32 (at most 65536 channels x 255 x 64
+// < 2^31).
+//
+// The bound is the one read of the buffer.  What kept an earlier form at 38% of
+// that was its instructions, 27 a sample: 16 samples a thread (so that the
+// overlap of 2^(K-1) - 1 samples cost as much as the samples themselves) and a
+// comparison and a mask bit per sample and width.  32 samples a thread and the
+// largest sum of each width (three-input max) take about 9 a sample: 3.25 ->
+// 1.46 ms for 8.22 GB (5.6 TB/s), and 1.05 -> 0.38 ms for 1.93 GB of integers.
+// A pulse's hits used to be written by the one or two threads that own its
+// samples (38 of the 47 us of a search of 13 MB with 7000 hits); through the
+// list all threads of the block share them: 8 us.  The staged tile is padded by 4 words after every 32: the
+// threads' 16-byte window loads then touch all banks evenly.
+constexpr int kPow2Threads = 128;
+constexpr int kPow2Per = 32;
+static_assert(kPow2Threads * kPow2Per == kSearchTile, "both search kernels use the same tiles");
+constexpr int kHitList = 1024;      // hits a block finishes per round
+
+__host__ __device__ __forceinline__ int spad32(int i) { return i + ((i >> 5) << 2); }
+
+__device__ __forceinline__ float max3(float a, float b, float c)
+{
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ __forceinline__ int32_t max3(int32_t a, int32_t b, int32_t c) { return __vimax3_s32(a, b, c); }
+
+// (a0, a1) + (b0, b1), each correctly rounded
+__device__ __forceinline__ void add2(float &a0, float &a1, float b0, float b1)
+{
+    asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %3};\n\tadd.rn.f32x2 a, a, b;\n\t"
+        "mov.b64 {%0, %1}, a;\n\t}"
+        : "+f"(a0), "+f"(a1) : "f"(b0), "f"(b1));
+}
+__device__ __forceinline__ void add2(int32_t &a0, int32_t &a1, int32_t b0, int32_t b1) { a0 += b0; a1 += b1; }
+
+// B_w at xs[0 .. w) of the padded tile, w = 2^p, by the tree of the search.
+template <typename T, int P>
+__device__ __forceinline__ T tree_sum(const T *x, int i)
+{
+    if constexpr (P == 0) return x[spad32(i)];
+    else return tree_sum<T, P - 1>(x, i) + tree_sum<T, P - 1>(x, i + (1 << (P - 1)));
+}
+
+template <typename T, int K>
+__device__ __forceinline__ T tree_sum_p(const T *x, int i, int p)
+{
+    if constexpr (K == 1) return tree_sum<T, 0>(x, i);
+    else return p == K - 1 ? tree_sum<T, K - 1>(x, i) : tree_sum_p<T, K - 1>(x, i, p);
+}
+
 template <bool kInt, int K>
-__global__ void __launch_bounds__(kSearchThreads)
+__global__ void __launch_bounds__(kPow2Threads)
 search_pow2_kernel(const void *__restrict__ out_, int64_t nout, const int32_t *__restrict__ wsorted,
                    const SearchParams *__restrict__ prm, const RowParams *__restrict__ rp,
                    dd_candidate *__restrict__ cands, int64_t cap, unsigned long long *__restrict__ count)
 {
     using T = typename std::conditional<kInt, int32_t, float>::type;
     constexpr int W = 1 << (K - 1);                 // widest boxcar
-    constexpr int kWin = kSearchPer + W - 1;
+    constexpr int kWin = (kPow2Per + W + 3) / 4 * 4;   // samples of a window, and some that no test uses
     extern __shared__ __align__(16) unsigned char sraw[];
     __shared__ int sidx[K];
     __shared__ float thf[K];
     __shared__ long long thi[K];
+    __shared__ unsigned short list[kHitList];       // thread << 8 | sorted width << 5 | sample
+    __shared__ int nlist;
+    __shared__ unsigned long long first;
     T *x = reinterpret_cast<T *>(sraw);
     const int row = blockIdx.y;
     const int64_t t0 = (int64_t)blockIdx.x * kSearchTile;
     if (threadIdx.x < K) {
         const int o = wsorted[K + threadIdx.x];     // original index of sorted width 2^threadIdx.x
         sidx[threadIdx.x] = o;
-        thf[threadIdx.x] = rp ? rp[blockIdx.y].thr_f[o] : prm->thr_f[o];
-        thi[threadIdx.x] = rp ? rp[blockIdx.y].thr_i[o] : prm->thr_i[o];
+        thf[threadIdx.x] = rp ? rp[row].thr_f[o] : prm->thr_f[o];
+        thi[threadIdx.x] = rp ? rp[row].thr_i[o] : prm->thr_i[o];
     }
+    if (threadIdx.x == 0) nlist = 0;
     const T *src = reinterpret_cast<const T *>(out_) + (size_t)row * nout + t0;
     const int64_t avail = nout - t0;                // > 0
-    T r[kSearchPer];
+    {
+        T r[kPow2Per];
+        if (avail >= kSearchTile) {
 #pragma unroll
-    for (int q = 0; q < kSearchPer; ++q) {
-        const int i = q * kSearchThreads + threadIdx.x;
-        r[q] = i < avail ? src[i] : (T)0;
-    }
+            for (int q = 0; q < kPow2Per; ++q) r[q] = __ldcs(src + q * kPow2Threads + threadIdx.x);
+        } else {
 #pragma unroll
-    for (int q = 0; q < kSearchPer; ++q) x[spad(q * kSearchThreads + threadIdx.x)] = r[q];
-    if ((int)threadIdx.x < W - 1) {
-        const int i = kSearchTile + threadIdx.x;
-        x[spad(i)] = i < avail ? src[i] : (T)0;
-    }
-    __syncthreads();
-    const int base = threadIdx.x * kSearchPer;
-    if (base >= avail) return;
-    const int64_t rem = avail - base;               // samples from this thread's first one on
-    T b[kWin];
-#pragma unroll
-    for (int k = 0; k < kWin; ++k) b[k] = x[spad(base + k)];
-    // hits as bits p*16 + i (width 2^p, sample i): the unrolled loop stays
-    // compact; the rare appends run once below
-    unsigned long long hits[2] = {0ull, 0ull};
-#pragma unroll
-    for (int p = 0; p < K; ++p) {
-        const int w = 1 << p;
-        if (p > 0) {
-            // b[k] = B_{w/2}(k) -> B_w(k); ascending k reads b[k + w/2] before it changes
-#pragma unroll
-            for (int k = 0; k + w <= kWin; ++k) b[k] = b[k] + b[k + w / 2];
-        }
-        unsigned m = 0;
-#pragma unroll
-        for (int i = 0; i < kSearchPer; ++i) {
-            bool hit;
-            if constexpr (kInt) hit = (long long)b[i] > thi[p];
-            else hit = b[i] > thf[p];
-            m |= (unsigned)hit << i;
-        }
-        const int64_t lim = rem - w + 1;            // tests with t + w <= nout
-        if (lim < kSearchPer) m &= lim > 0 ? (1u << lim) - 1u : 0u;
-        hits[p >> 2] |= (unsigned long long)m << (16 * (p & 3));
-    }
-#pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
-        unsigned long long bits = hits[h];
-        while (bits) {
-            const int bit = __ffsll((long long)bits) - 1;
-            bits &= bits - 1;
-            const int p = 4 * h + (bit >> 4), i = bit & 15, w = 1 << p;
-            // B_w(i) again, by the same pairwise tree (bit-identical value)
-            T v[1 << (K - 1)];
-            for (int q = 0; q < w; ++q) v[q] = x[spad(base + i + q)];
-            for (int d = 1; d < w; d *= 2)
-                for (int q = 0; q + d < w; q += 2 * d) v[q] = v[q] + v[q + d];
-            const unsigned long long pos = atomicAdd(count, 1ull);
-            if ((int64_t)pos < cap) {
-                dd_candidate c;
-                c.dm_idx = row; c.width_idx = sidx[p]; c.t = t0 + base + i;
-                c.snr = 0.f; c.reserved = 0.f; c.value = (double)v[0];
-                cands[pos] = c;
+            for (int q = 0; q < kPow2Per; ++q) {
+                const int i = q * kPow2Threads + threadIdx.x;
+                r[q] = i < avail ? __ldcs(src + i) : (T)0;
             }
         }
+        const int i = kSearchTile + threadIdx.x;
+        if ((int)threadIdx.x < W) x[spad32(i)] = i < avail ? src[i] : (T)0;
+#pragma unroll
+        for (int q = 0; q < kPow2Per; ++q) x[spad32(q * kPow2Threads + threadIdx.x)] = r[q];
+    }
+    __syncthreads();
+    const int base = threadIdx.x * kPow2Per;
+    const T *xb = x + spad32(base);
+    bool hit = false;
+    {
+        T b[kWin];
+#pragma unroll
+        for (int k = 0; k < kWin; k += 4) {
+            const int4 v = *reinterpret_cast<const int4 *>(xb + spad32(k));
+            if constexpr (kInt) { b[k] = v.x; b[k + 1] = v.y; b[k + 2] = v.z; b[k + 3] = v.w; }
+            else {
+                b[k] = __int_as_float(v.x); b[k + 1] = __int_as_float(v.y);
+                b[k + 2] = __int_as_float(v.z); b[k + 3] = __int_as_float(v.w);
+            }
+        }
+#pragma unroll
+        for (int p = 0; p < K; ++p) {
+            const int w = 1 << p;
+            // b[k] = B_{w/2}(k) -> B_w(k); ascending k reads b[k + w/2] before it changes
+            if (p == 1) {
+#pragma unroll
+                for (int k = 0; k + w <= kWin; ++k) b[k] = b[k] + b[k + 1];
+            } else if (p > 1) {
+#pragma unroll
+                for (int k = 0; k + w < kWin; k += 2) add2(b[k], b[k + 1], b[k + w / 2], b[k + 1 + w / 2]);
+            }
+            T m0 = b[0], m1 = b[1];
+#pragma unroll
+            for (int i = 2; i < kPow2Per - 2; i += 4) {
+                m0 = max3(m0, b[i], b[i + 1]);
+                m1 = max3(m1, b[i + 2], b[i + 3]);
+            }
+            m0 = max3(m0, m1, b[kPow2Per - 2]);
+            m1 = b[kPow2Per - 1];
+            if constexpr (kInt) hit |= (long long)m0 > thi[p] || (long long)m1 > thi[p];
+            else hit |= m0 > thf[p] || m1 > thf[p];
+        }
+    }
+    if (!__syncthreads_or(hit)) return;
+
+    // Runs with a hit again, sample by sample; their hits through the list, so
+    // that a pulse's hits, which lie in one or two runs, are finished by all
+    // threads of the block.
+    unsigned hits[K];
+#pragma unroll
+    for (int p = 0; p < K; ++p) hits[p] = 0u;
+    if (hit) {
+        const int64_t rem = avail - base;           // samples from this thread's first one on
+        T b[kWin];
+#pragma unroll
+        for (int k = 0; k < kWin; ++k) b[k] = xb[spad32(k)];
+#pragma unroll
+        for (int p = 0; p < K; ++p) {
+            const int w = 1 << p;
+            if (p > 0) {
+#pragma unroll
+                for (int k = 0; k + w <= kWin; ++k) b[k] = b[k] + b[k + w / 2];
+            }
+            unsigned m = 0;
+#pragma unroll
+            for (int i = 0; i < kPow2Per; ++i) {
+                bool h;
+                if constexpr (kInt) h = (long long)b[i] > thi[p];
+                else h = b[i] > thf[p];
+                m |= (unsigned)h << i;
+            }
+            const int64_t lim = rem - w + 1;        // tests with t + w <= nout
+            if (lim < kPow2Per) m &= lim > 0 ? (1u << lim) - 1u : 0u;
+            hits[p] = m;
+        }
+    }
+    for (;;) {
+        int mine = 0;
+#pragma unroll
+        for (int p = 0; p < K; ++p) mine += __popc(hits[p]);
+        int at = mine ? atomicAdd(&nlist, mine) : 0;
+#pragma unroll
+        for (int p = 0; p < K; ++p)
+            while (hits[p] && at < kHitList) {
+                list[at++] = (unsigned short)(threadIdx.x << 8 | p << 5 | (__ffs((int)hits[p]) - 1));
+                hits[p] &= hits[p] - 1;
+                --mine;
+            }
+        __syncthreads();
+        const int n = min(nlist, kHitList);
+        if (threadIdx.x == 0) first = atomicAdd(count, (unsigned long long)n);
+        __syncthreads();
+        for (int q = threadIdx.x; q < n; q += kPow2Threads) {
+            const int code = list[q], p = code >> 5 & 7, i = (code >> 8) * kPow2Per + (code & 31);
+            const T v = tree_sum_p<T, K>(x, i, p);   // B_w(i) again, by the same tree (the same value)
+            put_candidate(cands, cap, first + q, row, 1 << p, sidx[p], t0 + i, (double)v, prm, rp);
+        }
+        if (threadIdx.x == 0) nlist = 0;
+        if (!__syncthreads_or(mine > 0)) return;
     }
 }
 
 template <bool kInt, int K>
 static void launch_search_pow2(dim3 grid, cudaStream_t s, const void *out, const dd_plan *p)
 {
-    const size_t smem = (size_t)(spad(kSearchTile + (1 << (K - 1)) - 1) + 1) * 4;
-    search_pow2_kernel<kInt, K><<<grid, kSearchThreads, smem, s>>>(out, p->nsamp_out, p->d_wsorted, p->d_params,
+    const size_t smem = (size_t)spad32(kSearchTile + kPow2Per + (1 << (K - 1)) + 4) * 4;
+    search_pow2_kernel<kInt, K><<<grid, kPow2Threads, smem, s>>>(out, p->nsamp_out, p->d_wsorted, p->d_params,
                                                                     p->row_stats ? p->d_rowprm : nullptr,
                                                                     p->d_cands, p->cand_cap, p->d_count);
 }
@@ -632,20 +805,6 @@ int boundary_search_launch(dd_plan *p, const void *tail, const void *out, int L,
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "launch boundary_search_kernel");
     return DD_OK;
-}
-
-// S/N of the compacted hits: (B_w - w*mu) / (sigma*sqrt(w)), in double.
-__global__ void cand_snr_kernel(dd_candidate *__restrict__ cands, const unsigned long long *__restrict__ count,
-                                int64_t cap, const int32_t *__restrict__ widths, const SearchParams *__restrict__ prm,
-                                const RowParams *__restrict__ rp)
-{
-    const int64_t n = min((int64_t)*count, cap);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double w = (double)widths[cands[i].width_idx];
-        const double mu = rp ? rp[cands[i].dm_idx].mu : prm->mu;
-        const double sg = rp ? rp[cands[i].dm_idx].sigma : prm->sigma;
-        cands[i].snr = (float)((cands[i].value - w * mu) / (sg * sqrt(w)));
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -799,12 +958,13 @@ int search_launch(dd_plan *p, const void *out, cudaStream_t s)
     const bool isint = p->dtype == DD_U8;
     // widths are stored original-order in [0,nw) of d_wsorted's tail region
     const int32_t *w_orig = p->d_wsorted + 2 * p->nwidths;
+    const unsigned nfin = (unsigned)std::max<int64_t>(1, std::min<int64_t>(kFinBlocks, (p->n_partials + kFinRun - 1) / kFinRun));
     if (isint)
-        finalize_kernel<true><<<1, kFinThreads, 0, s>>>(p->d_partials, p->n_partials, w_orig,
-                                                        p->nwidths, p->sigma_k, p->d_params);
+        finalize_kernel<true><<<nfin, kFinThreads, 0, s>>>(p->d_partials, p->n_partials, w_orig, p->nwidths,
+                                                           p->sigma_k, p->d_params, p->d_count, p->d_fin);
     else
-        finalize_kernel<false><<<1, kFinThreads, 0, s>>>(p->d_partials, p->n_partials, w_orig,
-                                                         p->nwidths, p->sigma_k, p->d_params);
+        finalize_kernel<false><<<nfin, kFinThreads, 0, s>>>(p->d_partials, p->n_partials, w_orig, p->nwidths,
+                                                            p->sigma_k, p->d_params, p->d_count, p->d_fin);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "launch finalize_kernel");
     const RowParams *rp = nullptr;
@@ -819,8 +979,6 @@ int search_launch(dd_plan *p, const void *out, cudaStream_t s)
         if (e != cudaSuccess) return cuda_fail(e, "launch row_stats_kernel");
         rp = p->d_rowprm;
     }
-    e = cudaMemsetAsync(p->d_count, 0, sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return cuda_fail(e, "memset count");
     int wmax = 0;
     for (int w : p->widths) wmax = std::max(wmax, w);
     const int64_t ntile = (p->nsamp_out + kSearchTile - 1) / kSearchTile;
@@ -840,9 +998,6 @@ int search_launch(dd_plan *p, const void *out, cudaStream_t s)
                                                                 p->d_count);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "launch search_kernel");
-    cand_snr_kernel<<<64, 256, 0, s>>>(p->d_cands, p->d_count, p->cand_cap, w_orig, p->d_params, rp);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "launch cand_snr_kernel");
     return DD_OK;
 }
 
