@@ -307,6 +307,19 @@ DD_API int dd_share_tables(const int32_t *delays, int32_t ndm, int32_t nchans, d
                            int32_t config, int32_t *info, int32_t *rec_out, int64_t rec_cap, int32_t *base_out,
                            int64_t base_cap);
 
+/* The tables that configuration 12 runs with (host only), for inspection and
+ * tests: subbands of 4 or, where they move fewer shared-memory words, of 8
+ * channels; for DD_U8 the partial sums are counted in quads of four and read
+ * as pairs.  info[8] = dd_share_tables' six words, channels per subband, 1 if
+ * packed.  Records as dd_share_tables' with info[6] offsets per pattern (each
+ * pattern a whole number of 16-byte units); packed: pattern ends and starts in
+ * quads, offsets such that quad e's first term is staged element offset + 4e,
+ * a trial's index the word of its first pair (pairs from even sums in the
+ * first half of pmax words, from odd sums in the second). */
+DD_API int dd_share_ws_tables(const int32_t *delays, int32_t ndm, int32_t nchans, double foff, int32_t dtype,
+                              int32_t *info, int32_t *rec_out, int64_t rec_cap, int32_t *base_out,
+                              int64_t base_cap);
+
 /* Tile configuration the persistent launch uses (-1 if no beam uses it),
  * number of work items, and number of beams run by their own launch.  A new
  * batch starts with the first of configurations 9, 5, 3, 6, 4, 1, 0, 2 that

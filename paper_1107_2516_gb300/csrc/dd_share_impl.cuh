@@ -32,6 +32,8 @@
 
 #include "dd_lane_impl.cuh"
 
+#include <type_traits>
+
 namespace dd {
 
 // Table record of one (DM block, subband), int32 (16-byte multiple):
@@ -47,14 +49,17 @@ namespace dd {
 // the stage's rows (b_c = c * rs + the row offset of the pattern's first
 // sample minus start_p); rows_p = the rows of 32 sums before pattern p (the
 // patterns' sums are cut into rows of 32, each row inside one pattern).
+// Records of packed sums (uint8 input in the warp-specialised shape) have the
+// same layout and count P in quads of four sums: start_p, end_p and rows of 32
+// are in quads, staged element b_c + 4 e is channel c's term of quad e's first
+// sum, and q_j is the word that holds trial j's first pair (see the kernel).
 template <int CS, int NPMAX, int DB>
 struct ShareRec {
     static_assert(DB % 4 == 0, "trial offsets are loaded 4 at a time");
-    static_assert(CS + 3 <= 8, "pattern record: end, CS row offsets, start, rows before");
     static constexpr int kTrial = 0;
     static constexpr int kE = DB;
     static constexpr int kPat = DB + 4;                 // first pattern field (16-byte aligned)
-    static constexpr int kPatLen = 8;
+    static constexpr int kPatLen = (CS + 3 + 3) / 4 * 4;   // end, CS row offsets, start, rows before
     static constexpr int kPatStart = 1 + CS, kPatRows = 2 + CS;
     static constexpr int kMaxWarps = 8;
     static constexpr int kWarp = kPat + NPMAX * kPatLen;
@@ -77,6 +82,11 @@ struct ShareLaunch {
     int *err;
     size_t smem;
     int skew;              // 1: DM block b takes the time tiles in a rotated order (share_raster)
+    // warp-specialised shape
+    int cs;                // channels per subband: 4 or 8
+    int ns;                // input stages
+    int shifted;           // 1: rows start anywhere (in or pitch not 16-byte aligned)
+    int in_res;            // element of its 16-byte unit that `in` points at
 };
 
 // DM block / time tile of linear block index `lin`, as lane_raster, and with
@@ -108,8 +118,10 @@ __device__ __forceinline__ void share_raster(const ShareLaunch &a, int64_t lin, 
 // element row_start + l of each of its rows: whole rows RPS at a time with
 // the pattern's offsets set up once (every load of a step issued before its
 // stores), then the pattern's leftover rows in predicated steps of LRS rows.
+// xo[c] is added to channel c's staged elements (rows that start anywhere).
 template <typename Tin, typename R, int CS, int NW, int RPS = 4, int LRS = RPS>
-__device__ __forceinline__ void share_stage1(const int32_t *rec, const Tin *srow, float *Pb, int warp, int lane)
+__device__ __forceinline__ void share_stage1(const int32_t *rec, const Tin *srow, float *Pb, int warp, int lane,
+                                             const int (&xo)[CS])
 {
     static_assert(NW <= R::kMaxWarps, "stage-1 split recorded for at most kMaxWarps warps");
     int r = rec[R::kWarp + warp];
@@ -130,7 +142,7 @@ __device__ __forceinline__ void share_stage1(const int32_t *rec, const Tin *srow
         const int e0 = pst - (pexcl << 5) + lane;
         int src[CS];                                                   // staged element of channel c at e0
 #pragma unroll
-        for (int c = 0; c < CS; ++c) src[c] = b[1 + c] + e0;
+        for (int c = 0; c < CS; ++c) src[c] = b[1 + c] + xo[c] + e0;
         for (; r + RPS <= rfull; r += RPS) {
             // all RPS x CS loads before the RPS stores: the staged rows and P
             // are both shared memory, so the compiler may not move a store
@@ -169,6 +181,93 @@ __device__ __forceinline__ void share_stage1(const int32_t *rec, const Tin *srow
                 if (in[u]) Pb[e0 + ((r + u) << 5)] = v;
             }
         }
+        r = rend;
+        ++p;
+    }
+}
+
+// Stage 1 on bytes: lane l sums the four consecutive sums (a quad) of element
+// l of each of its rows of 32 quads.  Channel c's four bytes start anywhere in
+// a word: two word loads, one funnel shift, and their even and odd bytes are
+// added as pairs of 16-bit sums (at most 8 x 255).  Stage 2 reads pairs of
+// sums (u, u + 1) at any u, so P is stored twice, as pairs from even u (Pe)
+// and from odd u (Po); the pair that ends in the next quad takes that quad's
+// first sum from the bytes behind the four, one permute per two channels.
+// Per quad and lane 2 CS + 4 shared words for four sums, against 4 (CS + 1)
+// with one byte load (and a conversion to float) per term; stage 2 reads half
+// the words.  Bound by instructions, no longer by shared memory (ncu: issue
+// 71%, shared-memory wavefronts 60% of their peaks).  LOFAR-like beam of 2^18
+// uint8 samples, 2000 trials: 30.0 -> 20.7 ms; 4096 channels x 65536 samples,
+// 1500 trials: 24.7 -> 14.1 ms.  A single step where one row is left instead of a pair,
+// and the high half added with one dp2a instead of a shift and an add, are
+// 1.10x of that.
+template <typename R, int CS, int NW>
+__device__ __forceinline__ void share_stage1_bytes(const int32_t *rec, const uint8_t *srow, uint32_t *Pe, uint32_t *Po,
+                                                   int warp, int lane, const int (&xo)[CS])
+{
+    static_assert(NW <= R::kMaxWarps, "stage-1 split recorded for at most kMaxWarps warps");
+    constexpr uint32_t kEven = 0x00ff00ffu;
+    const uint32_t *words = reinterpret_cast<const uint32_t *>(srow);
+    int r = rec[R::kWarp + warp];
+    const int r1 = rec[R::kWarp + warp + 1];
+    int p = rec[R::kWarp + R::kMaxWarps + 1 + warp];
+    while (r < r1) {
+        const int32_t *pr = rec + R::kPat + p * R::kPatLen;
+        int b[R::kPatLen];
+#pragma unroll
+        for (int v = 0; v < R::kPatLen; v += 4) {
+            const int4 x = *reinterpret_cast<const int4 *>(pr + v);
+            b[v] = x.x; b[v + 1] = x.y; b[v + 2] = x.z; b[v + 3] = x.w;
+        }
+        const int pend = b[0], pst = b[R::kPatStart], pexcl = b[R::kPatRows];
+        const int rend = min(r1, pexcl + ((pend - pst + 31) >> 5));
+        int g = pst + ((r - pexcl) << 5) + lane;               // this lane's quad of row r
+        int src[CS];                                            // its first word of each channel, at g = 0
+        uint32_t sh[CS], sel[CS / 2];
+#pragma unroll
+        for (int c = 0; c < CS; ++c) {
+            const int e = b[1 + c] + xo[c];
+            src[c] = e >> 2;
+            sh[c] = (uint32_t)e << 3;                           // funnel shifts take it modulo 32
+        }
+#pragma unroll
+        for (int c = 0; c < CS; c += 2)                         // the bytes behind the four
+            sel[c / 2] = ((b[1 + c] + xo[c]) & 3) | (((b[2 + c] + xo[c + 1]) & 3) << 8) | 0x400;
+        // kRows rows from row r on, all loads before the first store.  Lanes past
+        // the pattern's end load too, at most 132 bytes behind the staged
+        // rows: records and slots follow them.
+        auto rows = [&](auto n) {
+            constexpr int kRows = decltype(n)::value;
+            uint32_t lo[kRows][CS], hi[kRows][CS];
+#pragma unroll
+            for (int u = 0; u < kRows; ++u)
+#pragma unroll
+                for (int c = 0; c < CS; ++c) {
+                    lo[u][c] = words[src[c] + g + 32 * u];
+                    hi[u][c] = words[src[c] + g + 32 * u + 1];
+                }
+#pragma unroll
+            for (int u = 0; u < kRows; ++u) {
+                uint32_t ev = 0, od = 0, nx = 0;
+#pragma unroll
+                for (int c = 0; c < CS; ++c) {
+                    const uint32_t x = __funnelshift_r(lo[u][c], hi[u][c], sh[c]);
+                    ev += x & kEven;
+                    od += __byte_perm(x, 0u, 0x4341);
+                }
+#pragma unroll
+                for (int c = 0; c < CS; c += 2) nx += __byte_perm(hi[u][c], hi[u][c + 1], sel[c / 2]) & kEven;
+                nx += nx >> 16;
+                if (u + 1 < kRows || g + 32 * u < pend) {       // only the last row can be partial
+                    const int w = 2 * (g + 32 * u);
+                    *reinterpret_cast<uint2 *>(Pe + w) = make_uint2(__byte_perm(ev, od, 0x5410), __byte_perm(ev, od, 0x7632));
+                    *reinterpret_cast<uint2 *>(Po + w) = make_uint2(__byte_perm(od, ev, 0x7610), __byte_perm(od, nx, 0x5432));
+                }
+            }
+        };
+        constexpr int kStep = CS == 4 ? 2 : 1;                  // 16 loads a step
+        for (; r + kStep <= rend; r += kStep, g += 32 * kStep) rows(std::integral_constant<int, kStep>());
+        if (r < rend) rows(std::integral_constant<int, 1>());
         r = rend;
         ++p;
     }
@@ -222,6 +321,35 @@ __device__ __forceinline__ void share_store(const ShareLaunch &a, const float (&
             for (int i = 0; i < TI; ++i) {
                 const int64_t t = t0 + lane + 32 * i;
                 if (dm < a.ndm && t < nout) { const float d = acc[j][i] - m; st.q += d * d; }
+            }
+        }
+    }
+}
+
+// The same for sums kept as pairs (packed stage 2): lane l's pair i holds the
+// samples t0 + 2 l + 64 i and the next one; a = low + 2^16 high and h = high
+// of the pair, modulo 2^32.
+template <int TI, int DR>
+__device__ __forceinline__ void share_store_pairs(const ShareLaunch &a, const uint32_t (&s)[DR][TI / 2],
+                                                  const uint32_t (&h)[DR][TI / 2], int dmw, int64_t t0, int lane,
+                                                  ShareStat<true> &st)
+{
+    int32_t *out = reinterpret_cast<int32_t *>(a.out);
+#pragma unroll
+    for (int j = 0; j < DR; ++j) {
+        const int dm = dmw + j;
+        if (dm >= a.ndm) break;
+        int32_t *row = out + (size_t)dm * a.nout;
+#pragma unroll
+        for (int i = 0; i < TI / 2; ++i) {
+            const uint32_t v[2] = {s[j][i] - (h[j][i] << 16), h[j][i]};
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int64_t t = t0 + 2 * lane + 64 * i + e;
+                if (t < a.nout) {
+                    __stcs(row + t, (int32_t)v[e]);
+                    st.n++; st.s += v[e]; st.q += (unsigned long long)v[e] * v[e];
+                }
             }
         }
     }
@@ -324,7 +452,8 @@ __device__ __forceinline__ bool share_tile(const ShareLaunch &a, int blk, int64_
         const Tin *srow = rows + (size_t)buf * stage_elems;
         float *Pb = P + (size_t)(s & 1) * a.pmax;
         // stage 1: every pattern's partial sum over the samples its trials need
-        share_stage1<Tin, R, CS, NW>(rec, srow, Pb, warp, lane);
+        const int xo[CS] = {};
+        share_stage1<Tin, R, CS, NW>(rec, srow, Pb, warp, lane, xo);
         // this warp's trials: index of their t = t0 term in P
 #pragma unroll
         for (int j = 0; j < DR; j += 4) {
@@ -501,61 +630,86 @@ __device__ __forceinline__ void group_stat_flush(const ShareLaunch &a, const Sha
 // launch allocation (checked on the host against the compiled register count
 // before the shape is used: an increase the block cannot cover would wait
 // forever).
-constexpr int kWsAccRegs = 168;
+constexpr int kWsAccRegs = 160;      // stage-2 warps: 128 accumulators
+constexpr int kWsStageRegs = 32;     // staging warps
+constexpr int kWsStage = 4;          // staging warps: a warpgroup
 template <int NW, int PW>
 struct WsRegs {
-    static constexpr int kThreads = (NW + PW) * 32;
-    static constexpr int kLaunch = (65536 / kThreads) / 8 * 8 > 255 ? 248 : (65536 / kThreads) / 8 * 8;
-    static constexpr bool kSplit = kLaunch < kWsAccRegs;
-    // stage-1 warps' share: what the launch leaves after the stage-2 warps' 168,
-    // 8 registers short of the most that would fit (slack for the compiled count)
-    static constexpr int kProd = kSplit ? ((NW + PW) * kLaunch - NW * kWsAccRegs) / PW / 8 * 8 - 8 : kLaunch;
-    static_assert(!kSplit || (kProd >= 24 && kProd % 8 == 0), "stage-1 warps need at least 24 registers");
-    static_assert(!kSplit || (PW % 4 == 0 && NW % 4 == 0), "setmaxnreg acts on whole warpgroups");
+    static constexpr int kWarps = NW + PW + kWsStage;
+    static constexpr int kLaunch = (65536 / (kWarps * 32)) / 8 * 8;
+    static constexpr int kProd = (kWarps * kLaunch - NW * kWsAccRegs - kWsStage * kWsStageRegs) / PW / 8 * 8;
+    static_assert(kLaunch < kWsAccRegs && kProd >= 24 && kProd <= kLaunch, "the stage-2 warps take registers from the others");
+    static_assert(PW % 4 == 0 && NW % 4 == 0 && kWsStage % 4 == 0, "setmaxnreg acts on whole warpgroups");
     // the compiled register count per thread the split needs
-    static constexpr int kNeed = kSplit ? (PW * kProd + NW * kWsAccRegs + NW + PW - 1) / (NW + PW) : 0;
+    static constexpr int kNeed = (kWsStage * kWsStageRegs + PW * kProd + NW * kWsAccRegs + kWarps - 1) / kWarps;
+    static_assert(kNeed <= kLaunch, "the shares stay within the launch's registers");
 };
+
+// Whether the phase has completed, without waiting.
+__device__ __forceinline__ bool mbar_done(uint64_t *bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(smem_addr(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
 
 // Kernel 5, warp-specialised: the same two stages on separate warps.  Warps
 // [0, PW) form subband s's partial sums (stage 1) into P slot s % PB and copy
 // the block's trial offsets next to them; warps [PW, PW + NW) add slot s into
-// their trials' accumulators (stage 2).  Hand-offs are mbarriers, not a block
-// barrier per subband:
-//   full[i]   input stage i has landed (TMA transaction bytes),
+// their trials' accumulators (stage 2); the last four stage the input.
+// Hand-offs are mbarriers, not a block barrier per subband:
+//   full[i]   input stage i has landed,
 //   empty[i]  every stage-1 warp is done with input stage i,
 //   pfull[b]  every stage-1 warp has written slot b,
 //   pempty[b] every stage-2 warp has read slot b,
-// so stage 1 runs up to PB - 1 subbands ahead of stage 2 and the two keep the
-// shared-memory pipe busy together.  Lane 0 of warp 0 issues the input copies
-// NS - 1 subbands ahead: at the top of subband s, those of subband s + NS - 1
-// into the stage subband s - 1 used, once every stage-1 warp is done with it.
+// so stage 1 runs up to PB - 1 subbands ahead of stage 2, the staging up to ns
+// ahead of stage 1, and the two stages keep the shared-memory pipe busy together.
+//
+// A thread that issues a bulk copy is held 250 to 300 cycles, whatever the
+// copy's size (clock64 around the issue).  When lane 0 of a stage-1 warp issued
+// the 5 copies of a subband it took 1277 of the subband's 2546 cycles on the
+// LOFAR-like plan, and everything waited for that warp's rows.  Four warps of
+// their own issue 1 to 3 copies each and are never waited for (626 of 2361
+// cycles; 888 of 2895 with 8 rows).  Measured against it: 16-byte cp.async by
+// the stage-2 threads (731 cycles a subband on the critical side) or by the
+// staging warps (1102; the copies then also take the loads' path into shared
+// memory: 31.9 against 30.5 ms on a quarter of the LOFAR-like plan).
 // One block per SM: NW * DR trials x 32 * TI samples of accumulators take
 // most of the register file, the stage-1 warps the rest.
 // Every wait is bounded; a warp whose wait gives up stops, the others then
-// give up on theirs, and the issuing thread waits (bounded) for its copies
-// still in flight before it returns.
-template <typename Tin, bool kInt, int TI, int DR, int NW, int PW, int CS, int NPMAX, int NS, int PB>
-__global__ void __launch_bounds__((NW + PW) * 32, 1) share_ws_kernel(ShareLaunch a)
+// give up on theirs, and the staging warps wait (bounded) for their copies still
+// in flight before they return.
+//
+// kAny: rows that start anywhere (in or pitch not 16-byte aligned).  Channel
+// c's copy starts res(c) elements early, at the 16-byte unit that holds its
+// first element, and ends with the unit of its last one, in a staged row one
+// unit longer; stage 1 reads res(c) elements on.
+template <typename Tin, bool kInt, int TI, int DR, int NW, int PW, int CS, int NPMAX, int PB, bool kAny>
+__global__ void __launch_bounds__((NW + PW + kWsStage) * 32, 1) share_ws_kernel(ShareLaunch a)
 {
     using Regs = WsRegs<NW, PW>;
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr int kDmBlk = DR * NW;
     using R = ShareRec<CS, NPMAX, kDmBlk>;
-    static_assert(NS >= 2 && PB >= 2, "input ring and slot ring need two entries");
+    static_assert(PB >= 2, "the slot ring needs two entries");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int rs = a.rs, nsub = a.nsub;
+    const int rs = a.rs, nsub = a.nsub, ns = a.ns;
 
-    // layout: [NS][CS][rs] Tin rows | [NS][kLen] int32 records |
+    // layout: [ns][CS][rs] Tin rows | [ns][kLen] int32 records |
     //         [PB] slots {int32 q[kDmBlk], float P[pmax]} | mbarriers at bar_off
     const size_t stage_elems = (size_t)CS * rs;
     Tin *rows = reinterpret_cast<Tin *>(smem);
-    int32_t *srec = reinterpret_cast<int32_t *>(smem + NS * stage_elems * sizeof(Tin));
-    int32_t *slots = srec + NS * R::kLen;
-    const size_t slot_len = (size_t)kDmBlk + a.pmax;
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem + a.bar_off);
-    uint64_t *empty = full + NS, *pfull = full + 2 * NS, *pempty = full + 2 * NS + PB;
+    int32_t *srec = reinterpret_cast<int32_t *>(smem + ns * stage_elems * sizeof(Tin));
+    int32_t *slots = srec + ns * R::kLen;
+    const size_t slot_len = (size_t)kDmBlk + a.pmax;      // packed sums: two halves of pmax / 2 words
+    uint64_t *pfull = reinterpret_cast<uint64_t *>(smem + a.bar_off);
+    uint64_t *pempty = pfull + PB, *full = pfull + 2 * PB, *empty = full + ns;
     if (tid == 0) {
-        for (int i = 0; i < NS; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], PW); }
+        for (int i = 0; i < ns; ++i) { mbar_init(&full[i], kWsStage); mbar_init(&empty[i], PW); }
         for (int b = 0; b < PB; ++b) { mbar_init(&pfull[b], PW); mbar_init(&pempty[b], NW); }
         mbar_fence_init();
     }
@@ -564,97 +718,120 @@ __global__ void __launch_bounds__((NW + PW) * 32, 1) share_ws_kernel(ShareLaunch
     int64_t t0;
     share_raster<TI>(a, blockIdx.x, blk, t0);
     t0 += a.t_base;
+    constexpr int kAl = 16 / (int)sizeof(Tin);
+    const int pitch_res = (int)(a.pitch & (kAl - 1));
+    auto res = [&](int c) { return (a.in_res + c * pitch_res) & (kAl - 1); };
 
     if (warp < PW) {
-        // ---- stage 1 (and the input copies)
-        if constexpr (Regs::kSplit) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(Regs::kProd));
-        const Tin *__restrict__ in = static_cast<const Tin *>(a.in);
-        const int32_t *brec = a.rec + (size_t)blk * nsub * R::kLen;
-        const int32_t *bbase = a.base + (size_t)blk * a.nchans;
-        const int32_t *blen = a.rlen + (size_t)blk * a.nchans;
-        auto row_bytes = [&](int b, int rl, int64_t &g) -> uint32_t {
-            g = t0 + b;
-            int64_t n = a.nsamp_in_al - g;
-            n = n < 0 ? 0 : (n > rl ? rl : n);
-            return (uint32_t)(n * (int64_t)sizeof(Tin));
-        };
-        int rb[CS], rl[CS];
-        auto load_rb = [&](int s) {
-#pragma unroll
-            for (int cc = 0; cc < CS; ++cc) { rb[cc] = bbase[s * CS + cc]; rl[cc] = blen[s * CS + cc]; }
-        };
-        auto issue = [&](int s) {
-            const int buf = s % NS;
-            uint32_t bytes = (uint32_t)(R::kLen * sizeof(int32_t));
-#pragma unroll
-            for (int cc = 0; cc < CS; ++cc) { int64_t g; bytes += row_bytes(rb[cc], rl[cc], g); }
-            mbar_arrive_tx(&full[buf], bytes);
-            bulk_g2s(srec + (size_t)buf * R::kLen, brec + (size_t)s * R::kLen, (uint32_t)(R::kLen * sizeof(int32_t)),
-                     &full[buf]);
-            const uint64_t pol = l2_evict_last();
-#pragma unroll
-            for (int cc = 0; cc < CS; ++cc) {
-                int64_t g;
-                const uint32_t nb = row_bytes(rb[cc], rl[cc], g);
-                if (nb)
-                    bulk_g2s_hint(rows + (size_t)buf * stage_elems + (size_t)cc * rs,
-                                  in + (size_t)(s * CS + cc) * a.pitch + g, nb, &full[buf], pol);
-            }
-        };
-        int issued = 0;   // copies issued (thread 0)
-        if (tid == 0) {
-            for (; issued < NS - 1 && issued < nsub; ++issued) { load_rb(issued); issue(issued); }
-            if (issued < nsub) load_rb(issued);
-        }
-        bool ok = true;
-        int s = 0;
-        for (; s < nsub; ++s) {
-            if (warp == 0) {
-                // refill the stage subband s - 1 used once every stage-1 warp is done with it
-                bool go = true;
-                if (lane == 0 && issued < nsub) {
-                    if (s >= 1) go = mbar_wait(&empty[(s - 1) % NS], (uint32_t)(((s - 1) / NS) & 1), a.err);
-                    if (go) {
-                        issue(issued);
-                        ++issued;
-                        if (issued < nsub) load_rb(issued);
-                    }
-                }
-                ok = __shfl_sync(0xffffffffu, go ? 1 : 0, 0) != 0;
-            }
-            const int pb = s % PB, ib = s % NS;
-            if (ok && s >= PB) ok = mbar_wait(&pempty[pb], (uint32_t)(((s / PB) - 1) & 1), a.err);
-            if (ok) ok = mbar_wait(&full[ib], (uint32_t)((s / NS) & 1), a.err);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
+        // ---- stage 1
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(Regs::kProd));
+        int ib = 0, pb = 0;                      // input stage, slot
+        uint32_t fpar = 0, epar = 1;             // their phases' parities (a fresh slot counts as read)
+        for (int s = 0; s < nsub; ++s) {
+            const bool e = mbar_done(&pempty[pb], epar), f = mbar_done(&full[ib], fpar);
+            bool ok = e && f;
+            if (!ok) ok = mbar_wait(&pempty[pb], epar, a.err) && mbar_wait(&full[ib], fpar, a.err);
+            if (!__all_sync(0xffffffffu, ok)) break;
             const int32_t *rec = srec + (size_t)ib * R::kLen;
+            const Tin *srow = rows + (size_t)ib * stage_elems;
             int32_t *slot = slots + (size_t)pb * slot_len;
-            // whole rows 8 per step (no accumulators here), leftovers 4 per step
-            share_stage1<Tin, R, CS, PW, 8, 4>(rec, rows + (size_t)ib * stage_elems,
-                                               reinterpret_cast<float *>(slot + kDmBlk), warp, lane);
+            int xo[CS] = {};
+            if constexpr (kAny) {
+#pragma unroll
+                for (int cc = 0; cc < CS; ++cc) xo[cc] = cc * kAl + res(s * CS + cc);   // the records' rows are one unit shorter
+            }
+            if constexpr (kInt) {
+                uint32_t *P = reinterpret_cast<uint32_t *>(slot + kDmBlk);
+                share_stage1_bytes<R, CS, PW>(rec, srow, P, P + a.pmax / 2, warp, lane, xo);
+            } else {
+                // 32 loads a step (no accumulators here): 8 or 4 whole rows; leftover rows in half steps
+                constexpr int kRows = 32 / CS;
+                share_stage1<Tin, R, CS, PW, kRows, kRows / 2>(rec, srow, reinterpret_cast<float *>(slot + kDmBlk), warp,
+                                                               lane, xo);
+            }
             if (warp == PW - 1)
                 for (int j = lane; j < kDmBlk; j += 32) slot[j] = rec[R::kTrial + j];
             __syncwarp();
             if (lane == 0) { mbar_arrive(&pfull[pb]); mbar_arrive(&empty[ib]); }
+            if (++pb == PB) { pb = 0; epar ^= 1u; }
+            if (++ib == ns) { ib = 0; fpar ^= 1u; }
+        }
+        return;
+    }
+
+    if (warp >= PW + NW) {
+        // ---- staging: warp w stages rows w, w + 4, .. of the subband, the last
+        // one its record too.  A row's start and length are loaded one
+        // subband early, by lane i for the warp's i-th row.
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kWsStageRegs));
+        constexpr int kRows = CS / kWsStage;       // rows per warp
+        const int w = warp - PW - NW, mine = w + kWsStage * min(lane, kRows - 1);
+        const Tin *in = static_cast<const Tin *>(a.in) + t0;
+        const int32_t *rb_p = a.base + (size_t)blk * a.nchans + mine, *rl_p = a.rlen + (size_t)blk * a.nchans + mine;
+        const int32_t *rec_p = a.rec + (size_t)blk * nsub * R::kLen;
+        const bool with_rec = w == kWsStage - 1;
+        const uint64_t pol = l2_evict_last();      // other DM blocks of this tile stage these rows soon
+        int rb = rb_p[0], rl = rl_p[0], ib = 0, s = 0;
+        uint32_t par = 1;                          // a fresh stage counts as done with
+        for (; s < nsub; ++s) {
+            if (!__all_sync(0xffffffffu, mbar_wait(&empty[ib], par, a.err))) break;
+            // lane i: its row's first element and 16-byte units
+            int64_t g = (int64_t)(s * CS + mine) * a.pitch + rb, n = a.nsamp_in_al - (t0 + rb);
+            n = n < 0 ? 0 : (n > rl ? rl : n);
+            if constexpr (kAny) {
+                const int d = res(s * CS + mine);
+                g -= d;
+                if (n > 0) n += d;
+            }
+            const int units = lane < kRows ? (int)((n + kAl - 1) / kAl) : 0;
+            if (s + 1 < nsub) { rb = rb_p[(s + 1) * CS]; rl = rl_p[(s + 1) * CS]; }
+            Tin *dst = rows + (size_t)ib * stage_elems + (size_t)w * rs;
+            int32_t *rdst = srec + (size_t)ib * R::kLen;
+            const int32_t *rsrc = rec_p + (size_t)s * R::kLen;
+            const int all = __reduce_add_sync(0xffffffffu, units);
+            if (lane == 0) mbar_arrive_tx(&full[ib], (uint32_t)(all * 16 + (with_rec ? R::kLen * 4 : 0)));
+#pragma unroll
+            for (int i = 0; i < kRows; ++i) {
+                const int64_t gi = __shfl_sync(0xffffffffu, g, i);
+                const int ui = __shfl_sync(0xffffffffu, units, i);
+                if (lane == 0 && ui)
+                    bulk_g2s_hint(dst + (size_t)(i * kWsStage) * rs, in + gi, (uint32_t)ui * 16, &full[ib], pol);
+            }
+            if (lane == 0 && with_rec) bulk_g2s(rdst, rsrc, R::kLen * 4, &full[ib]);
+            if (++ib == ns) { ib = 0; par ^= 1u; }
         }
         // after a wait gave up: let the copies still in flight land before leaving
-        if (tid == 0)
-            for (int u = s; u < issued; ++u) mbar_wait(&full[u % NS], (uint32_t)((u / NS) & 1), a.err);
+        if (lane == 0)
+            for (int u = max(0, s - ns); u < s; ++u) mbar_wait(&full[u % ns], (uint32_t)((u / ns) & 1), a.err);
         return;
     }
 
     // ---- stage 2: one shared word per add
-    if constexpr (Regs::kSplit) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kWsAccRegs));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kWsAccRegs));
+    // Packed sums: a word holds the sums of two consecutive samples, and is
+    // added whole (low + 2^16 high, modulo 2^32) and by its high half: the two
+    // sums follow exactly from the two accumulators, with one word per two adds.
     const int cw = warp - PW;
-    float acc[DR][TI];
+    float acc[kInt ? 1 : DR][kInt ? 1 : TI];
+    uint32_t pa[kInt ? DR : 1][kInt ? TI / 2 : 1], ph[kInt ? DR : 1][kInt ? TI / 2 : 1];
+    if constexpr (kInt) {
 #pragma unroll
-    for (int j = 0; j < DR; ++j)
+        for (int j = 0; j < DR; ++j)
 #pragma unroll
-        for (int i = 0; i < TI; ++i) acc[j][i] = 0.f;
+            for (int i = 0; i < TI / 2; ++i) { pa[j][i] = 0u; ph[j][i] = 0u; }
+    } else {
+#pragma unroll
+        for (int j = 0; j < DR; ++j)
+#pragma unroll
+            for (int i = 0; i < TI; ++i) acc[j][i] = 0.f;
+    }
+
     bool ok = true;
+    int pb = 0;
+    uint32_t ppar = 0;
     for (int s = 0; s < nsub; ++s) {
-        const int pb = s % PB;
-        ok = __all_sync(0xffffffffu, mbar_wait(&pfull[pb], (uint32_t)((s / PB) & 1), a.err));
+        ok = mbar_done(&pfull[pb], ppar) || mbar_wait(&pfull[pb], ppar, a.err);
+        ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         const int32_t *slot = slots + (size_t)pb * slot_len;
         const float *Pb = reinterpret_cast<const float *>(slot + kDmBlk);
@@ -666,39 +843,57 @@ __global__ void __launch_bounds__((NW + PW) * 32, 1) share_ws_kernel(ShareLaunch
         }
 #pragma unroll
         for (int j = 0; j < DR; ++j) {
-            const float *pp = Pb + q[j] + lane;
+            if constexpr (kInt) {
+                const uint32_t *pp = reinterpret_cast<const uint32_t *>(Pb) + q[j] + lane;
 #pragma unroll
-            for (int i = 0; i < TI; ++i) acc[j][i] += pp[32 * i];
+                for (int i = 0; i < TI / 2; ++i) {
+                    const uint32_t v = pp[32 * i];
+                    pa[j][i] += v;
+                    ph[j][i] = __dp2a_lo(v, 0x0100u, ph[j][i]);   // + its high half
+                }
+            } else {
+                const float *pp = Pb + q[j] + lane;
+#pragma unroll
+                for (int i = 0; i < TI; ++i) acc[j][i] += pp[32 * i];
+            }
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&pempty[pb]);
+        if (++pb == PB) { pb = 0; ppar ^= 1u; }
     }
     ShareStat<kInt> st;
-    if (ok) share_store<kInt, TI, DR>(a, acc, blk * kDmBlk + cw * DR, t0, lane, st);
+    if (ok) {
+        if constexpr (kInt) share_store_pairs<TI, DR>(a, pa, ph, blk * kDmBlk + cw * DR, t0, lane, st);
+        else share_store<kInt, TI, DR>(a, acc, blk * kDmBlk + cw * DR, t0, lane, st);
+    }
     group_stat_flush<kInt>(a, st, blockIdx.x, PW, NW);
 }
 
-// Compiled shapes: subbands of 4 channels, at most 16 patterns per (block,
-// subband); {samples per lane, DM trials per warp, warps (stage-2 warps in
-// the warp-specialised form), resident blocks per SM the register budget
-// targets, input stages, stage-1 warps (0: the one-barrier-per-subband
-// kernel, whose warps do both stages), partial-sum slots, stage-1 rows of
-// warp 0 in percent of another warp's (its first thread issues the input
-// copies, which hold it for ~1000 cycles per subband: a smaller share keeps
-// it from being the last one at each subband's barrier or hand-off)}.
+// Compiled shapes: subbands of 4 channels (the warp-specialised shape also 8),
+// at most 16 patterns per (block, subband); {samples per lane, DM trials per
+// warp, warps (stage-2 warps in the warp-specialised form), resident blocks
+// per SM the register budget targets, input stages (at most, in the
+// warp-specialised form), stage-1 warps (0: the one-barrier-per-subband
+// kernel, whose warps do both stages), partial-sum slots, stage-1 rows of warp
+// 0 in percent of another warp's (its first thread issues the one-barrier
+// kernels' input copies, which hold it for ~1000 cycles per subband: a smaller
+// share keeps it from being the last one at each subband's barrier.  The
+// warp-specialised kernel's split gives every stage-1 warp an equal share;
+// its value here only enters dd_share_tables' records)}.
 constexpr int kShCS = 4, kShNP = 16;
 struct ShareShape { int ti, dr, nw, minb, ns, pw, pb, w0; };
 constexpr int kNumShareCfg = 4;
+constexpr int kShareWs = 3;          // the warp-specialised shape
 constexpr ShareShape kShareCfg[kNumShareCfg] = {
-    {16, 8, 4, 3, 2, 0, 2, 70}, {8, 8, 4, 5, 2, 0, 2, 70}, {16, 8, 6, 2, 2, 0, 2, 70}, {16, 8, 8, 1, 3, 8, 3, 50}};
+    {16, 8, 4, 3, 2, 0, 2, 70}, {8, 8, 4, 5, 2, 0, 2, 70}, {16, 8, 6, 2, 2, 0, 2, 70}, {16, 8, 8, 1, 6, 8, 3, 50}};
 template <int DB>
 using ShareRecDB = ShareRec<kShCS, kShNP, DB>;
 
 cudaError_t share_launch(int k, dd_dtype t, const ShareLaunch &a, cudaStream_t s);
 cudaError_t share_prepare(int k, size_t optin);
-// false if shape k's kernels were compiled with fewer registers than its
-// register split needs (the shape is then not used)
-bool share_regs_ok(int k);
+// false if shape k's kernels for this input type were compiled with fewer
+// registers than their register split needs (they are then not used)
+bool share_regs_ok(int k, dd_dtype t);
 // Mixed persistent batch of kernel 5 shape 0 and kernel 3 shape 2 (the same
 // block geometry): grid = sms * that shape's resident blocks per SM.
 cudaError_t mixed_batch_launch(const LaneBatchLaunch &b, int sms, size_t smem, cudaStream_t s);

@@ -1,0 +1,61 @@
+"""Kernel 5's warp-specialised shape on the GPU where its forms differ:
+subbands of 4 and 8 channels, packed uint8 sums, rows that start anywhere,
+ragged last DM blocks and time tiles, against the oracle."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+import oracle  # noqa: E402
+import synth  # noqa: E402
+import paper_1107_2516_gb300 as dd  # noqa: E402
+from test_share_ws_tables import CASES, TYPE  # noqa: E402
+
+
+def run(x, off, pitch, d, m, nch, fch1, foff, ts, dms, nsamp, dtype):
+    flat = np.zeros(off + nch * pitch, x.dtype)
+    for c in range(nch):
+        flat[off + c * pitch:off + c * pitch + nsamp] = x[c]
+        flat[off + c * pitch + nsamp:off + (c + 1) * pitch] = 99
+    dev = torch.from_numpy(flat.view(np.int16) if dtype == "f16" else flat).cuda()
+    plan = dd.Plan(nch, fch1, foff, ts, dms, [1, 2, 4], 6.0, TYPE[dtype], nsamp)
+    assert plan.maxshift == m
+    plan.set_tile(12, 8)
+    out = torch.full((len(dms) * plan.nsamp_out + 64,), -7, dtype=torch.int32 if dtype == "u8" else torch.float32, device="cuda")
+    plan.execute(dev.data_ptr() + off * flat.itemsize, pitch, out)
+    _, _ = plan.search(out, allow_overflow=True)
+    mu, sg = plan.stats()
+    got = out.cpu().numpy()
+    plan.close()
+    assert np.all(got[-64:] == -7)
+    return got[:-64].reshape(len(dms), nsamp - m), mu, sg
+
+
+@pytest.mark.parametrize("dtype", ["f32", "u8", "f16"])
+@pytest.mark.parametrize("off,pad", [(0, None), (0, 1), (3, 5), (1, None)])
+@pytest.mark.parametrize("case", range(len(CASES)))
+def test_forms_against_oracle(case, off, pad, dtype):
+    nch, fch1, foff, ts, dms, nsamp, _ = CASES[case]
+    al = 16 // {"f32": 4, "u8": 1, "f16": 2}[dtype]
+    for n in (nsamp, nsamp + 511, nsamp + 1537):
+        d, m = oracle.delays(nch, fch1, foff, ts, dms)
+        pitch = n + pad if pad is not None else -(-n // al) * al
+        x = synth.noise_f32(nch, n, 7 + case)
+        x = synth.quantize_u8(x) if dtype == "u8" else x.astype(np.float16) if dtype == "f16" else x
+        got, mu, sg = run(x, off, pitch, d, m, nch, fch1, foff, ts, dms, n, dtype)
+        ref = oracle.dedisperse(x if dtype == "u8" else x.astype(np.float32), np.asarray(d), n - m)
+        if dtype == "u8":
+            assert np.array_equal(got, ref)
+        else:
+            assert np.max(np.abs(got - ref)) <= 1e-5 * nch
+        assert abs(mu - ref.mean()) <= 1e-5 * max(1.0, abs(ref.mean())) and abs(sg - ref.std()) <= 1e-5 * ref.std()
+
+
+def test_largest_bytes():
+    # every byte 255 in every channel of an 8-channel subband plan: the largest packed sums
+    nch, fch1, foff, ts, dms, nsamp, _ = CASES[2]
+    d, m = oracle.delays(nch, fch1, foff, ts, dms)
+    x = np.full((nch, nsamp), 255, np.uint8)
+    got, mu, _ = run(x, 0, nsamp + 4, d, m, nch, fch1, foff, ts, dms, nsamp, "u8")
+    assert np.all(got == 255 * nch) and mu == 255.0 * nch
