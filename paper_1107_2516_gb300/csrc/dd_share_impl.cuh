@@ -516,7 +516,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) mixed_batch_kernel(LaneBatchLau
     __shared__ int s_item;
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + b.bar_off), *sbar = bar + kStages;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kStages; ++s) mbar_init(&bar[s], 1);
+        for (int s = 0; s < kStages; ++s) mbar_init(&bar[s], NW);
         for (int s = 0; s < NS; ++s) mbar_init(&sbar[s], 1);
         mbar_fence_init();
     }

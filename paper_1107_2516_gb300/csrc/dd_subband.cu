@@ -89,54 +89,61 @@ __global__ void __launch_bounds__(NW * 32, 3) sub_kernel(SubLaunch a)
     const int nst = (nchans + ch - 1) / ch;
 
     if (tid == 0) {
-        for (int s = 0; s < kStages; ++s) mbar_init(&bar[s], 1);
+        for (int s = 0; s < kStages; ++s) mbar_init(&bar[s], NW);
         mbar_fence_init();
     }
     __syncthreads();
 
-    auto row_bytes = [&](int c, int64_t &g) -> uint32_t {
-        g = t0 + bbase[c];
-        int64_t n = a.nsamp_in_al - g;
-        n = n < 0 ? 0 : (n > rs ? rs : n);
-        return (uint32_t)(n * (int64_t)sizeof(Tin));
-    };
+    // Stage s's copies, spread over the warps as in kernel 3: lane l of warp w
+    // issues row w + NW l, the last warp the offsets too.
+    const int mine = warp + NW * lane;
+    int rb = mine < ch ? bbase[min(mine, nchans - 1)] : 0;   // of the next stage to issue
     auto issue = [&](int s) {
         const int buf = s % kStages;
         const int c0 = s * ch;
         const int cn = min(ch, nchans - c0);
-        uint32_t bytes = (uint32_t)(cn * kDmBlk * sizeof(int32_t));
-        for (int cc = 0; cc < cn; ++cc) { int64_t g; bytes += row_bytes(c0 + cc, g); }
-        mbar_arrive_tx(&bar[buf], bytes);
-        bulk_g2s(soffs + (size_t)buf * ch * kDmBlk, boffs + (size_t)c0 * kDmBlk,
-                 (uint32_t)(cn * kDmBlk * sizeof(int32_t)), &bar[buf]);
-        for (int cc = 0; cc < cn; ++cc) {
-            int64_t g;
-            const uint32_t nb = row_bytes(c0 + cc, g);
-            const int64_t r = (int64_t)B.in_row + (int64_t)(c0 + cc) * a.in_rstride;
-            if (nb)
-                bulk_g2s(rows + (size_t)buf * stage_elems + (size_t)cc * rs, in + r * a.pitch + g, nb,
-                         &bar[buf]);
+        const int64_t g = t0 + rb;
+        int64_t n = a.nsamp_in_al - g;
+        n = n < 0 || mine >= cn ? 0 : (n > rs ? rs : n);
+        const uint32_t nb = (uint32_t)(n * (int64_t)sizeof(Tin)), ob = (uint32_t)(cn * kDmBlk * sizeof(int32_t));
+        const uint32_t bytes = __reduce_add_sync(0xffffffffu, nb) + (warp == NW - 1 ? ob : 0u);
+        if (lane == 0) {
+            mbar_arrive_tx(&bar[buf], bytes);
+            if (warp == NW - 1) bulk_g2s(soffs + (size_t)buf * ch * kDmBlk, boffs + (size_t)c0 * kDmBlk, ob, &bar[buf]);
         }
+        __syncwarp();
+        if (nb) {
+            const int64_t r = (int64_t)B.in_row + (int64_t)(c0 + mine) * a.in_rstride;
+            bulk_g2s(rows + (size_t)buf * stage_elems + (size_t)mine * rs, in + r * a.pitch + g, nb, &bar[buf]);
+        }
+        if (mine < ch) rb = bbase[min(c0 + ch + mine, nchans - 1)];
     };
 
+    constexpr bool kBytes = std::is_same<Tin, uint8_t>::value;
     float acc[DR][TI];
+    ByteSums<kBytes ? TI : 4, kBytes ? DR : 4> bs;
+    if constexpr (kBytes) {
+        bs.clear();
+    } else {
 #pragma unroll
-    for (int j = 0; j < DR; ++j)
+        for (int j = 0; j < DR; ++j)
 #pragma unroll
-        for (int i = 0; i < TI; ++i) acc[j][i] = 0.f;
+            for (int i = 0; i < TI; ++i) acc[j][i] = 0.f;
+    }
 
-    if (tid == 0)
-        for (int s = 0; s < kStages - 1 && s < nst; ++s) issue(s);
+    for (int s = 0; s < kStages - 1 && s < nst; ++s) issue(s);
 
+    const bool idle = warp * DR >= B.ntr;         // none of the warp's trials exist
     bool ok = true;
     for (int s = 0; s < nst; ++s) {
-        if (tid == 0 && s + kStages - 1 < nst) issue(s + kStages - 1);
+        if (s + kStages - 1 < nst) issue(s + kStages - 1);
         const int buf = s % kStages;
         if (ok) ok = mbar_wait(&bar[buf], (uint32_t)((s / kStages) & 1), a.err);
-        const int cn = min(ch, nchans - s * ch);
+        const int cn = idle ? 0 : min(ch, nchans - s * ch);
         const Tin *srow = rows + (size_t)buf * stage_elems + lane;
         const int32_t *so = soffs + (size_t)buf * ch * kDmBlk + warp * DR;
-        for (int cc = 0; cc < cn; ++cc) {
+        if constexpr (kBytes) bs.add_stage(srow - lane, rs, so, kDmBlk, cn, lane);
+        else for (int cc = 0; cc < cn; ++cc) {
             const Tin *r = srow + (size_t)cc * rs;
             int o[DR];
 #pragma unroll
@@ -156,6 +163,14 @@ __global__ void __launch_bounds__(NW * 32, 3) sub_kernel(SubLaunch a)
     ok = __syncthreads_and(ok);
     if (!ok) return;
 
+    // this lane's sample i of the tile
+    auto sample = [&](int i) { return t0 + (kBytes ? 4 * lane + 128 * (i / 4) + i % 4 : lane + 32 * i); };
+    if constexpr (kBytes) {
+#pragma unroll
+        for (int j = 0; j < DR; ++j)
+#pragma unroll
+            for (int i = 0; i < TI; ++i) acc[j][i] = (float)bs.at(j, i / 4, i % 4);   // exact: below 2^24
+    }
     const int64_t nout = a.nout;
     if constexpr (kInt) {
         long long n = 0, s = 0;
@@ -166,7 +181,7 @@ __global__ void __launch_bounds__(NW * 32, 3) sub_kernel(SubLaunch a)
             const int jr = warp * DR + j;
 #pragma unroll
             for (int i = 0; i < TI; ++i) {
-                const int64_t t = t0 + lane + 32 * i;
+                const int64_t t = sample(i);
                 if (jr < B.ntr && t < nout) {
                     const long long v = __float2int_rn(acc[j][i]);
                     out[(size_t)(B.row0 + jr) * a.out_pitch + t] = (int32_t)v;
@@ -184,7 +199,7 @@ __global__ void __launch_bounds__(NW * 32, 3) sub_kernel(SubLaunch a)
             const int jr = warp * DR + j;
 #pragma unroll
             for (int i = 0; i < TI; ++i) {
-                const int64_t t = t0 + lane + 32 * i;
+                const int64_t t = sample(i);
                 if (jr < B.ntr && t < nout) {
                     out[(size_t)(B.row0 + jr) * a.out_pitch + t] = acc[j][i];
                     n++; s += acc[j][i];
@@ -199,7 +214,7 @@ __global__ void __launch_bounds__(NW * 32, 3) sub_kernel(SubLaunch a)
                 const int jr = warp * DR + j;
 #pragma unroll
                 for (int i = 0; i < TI; ++i) {
-                    const int64_t t = t0 + lane + 32 * i;
+                    const int64_t t = sample(i);
                     if (jr < B.ntr && t < nout) { const float d = acc[j][i] - m; q += d * d; }
                 }
             }
@@ -289,7 +304,11 @@ static int finish_stage(SubStage &st, long long need, size_t eb, size_t optin)
     st.rs = (int)((need + 15) / 16 * 16);
     const size_t budget = std::min<size_t>(optin, (228 * 1024) / 3 - 1024) - 1024;
     const size_t per_ch = (size_t)st.rs * eb + (size_t)st.db * sizeof(int32_t);
-    st.ch = (int)std::min<size_t>(16, budget / (kStages * per_ch));
+    // a block sums few channels (32 in the usual plans): 4 a stage, so that it
+    // starts on the first while the others land (stage 2 of the LOFAR-like
+    // plan 9.6 ms with 16 or 8 a stage, 8.2 with 4, which also lets a fourth
+    // block share the SM; stage 1 the same)
+    st.ch = (int)std::min<size_t>(4, budget / (kStages * per_ch));
     if (st.ch < 1) return set_error(DD_ERR_ARG, "subband rows too long for shared memory (%d samples)", st.rs);
     st.bar_off = (int)(((size_t)kStages * st.ch * per_ch + 15) / 16 * 16);
     st.smem = (size_t)st.bar_off + kStages * sizeof(uint64_t);
