@@ -54,3 +54,27 @@ def test_byte_sums_of_subbands(cs, ndm, group):
         ref = oracle.subband_dedisperse(np.ascontiguousarray(x[:, :nsamp]), d1, d2, group, nout)
         assert np.array_equal(out.cpu().numpy().reshape(ndm, nout), ref)
         plan.close()
+
+
+@pytest.mark.parametrize("bins", [(2,), (4,), (2, 4), (4, 2, 2), (8, 4, 2), (3, 2)])
+@pytest.mark.parametrize("extra,pad", [(0, 0), (1, 15), (2, 14), (3, 13), (5, 11), (2, 1)])
+def test_binning_remainders(bins, extra, pad):
+    # sums of bytes over 2, 4 or 8 are exact in float32, and so are their sums over the channels
+    nch, nsub, nsamp = 6, 2, 8192 + extra
+    rng = np.random.default_rng(extra)
+    x = rng.integers(0, 256, (nch, nsamp + pad)).astype(np.uint8)
+    passes = [(10.0 * i, 10.0 * i + 4.0, 1.0, b, 2.0) for i, b in enumerate(bins)]
+    plan = dd.SurveyPlan(nch, 150.0, -0.1, 1e-3, passes, nsub, [1], 6.0, dd.DD_U8, nsamp)
+    outs = [torch.empty(p[0] * p[4], device="cuda") for p in plan.passes]
+    plan.execute(torch.from_numpy(x).cuda(), nsamp + pad, outs)
+    for i, b in enumerate(bins):
+        xb = x[:, :nsamp // b * b].reshape(nch, -1, b).astype(np.float64).sum(2) / b
+        dms = plan.dm_list(i)
+        _, d1, d2, m = oracle.subband_tables(nch, 150.0, -0.1, 1e-3 * b, dms, 2, nsub)
+        ref = oracle.subband_dedisperse(xb.astype(np.float32), d1, d2, 2, xb.shape[1] - m)
+        got = outs[i].cpu().numpy().reshape(ref.shape)
+        if b == 3:
+            assert np.max(np.abs(got - ref)) <= 1e-5 * nch * 256
+        else:
+            assert np.array_equal(got, ref)
+    plan.close()
