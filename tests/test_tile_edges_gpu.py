@@ -78,3 +78,19 @@ def test_binning_remainders(bins, extra, pad):
         else:
             assert np.array_equal(got, ref)
     plan.close()
+
+
+@pytest.mark.parametrize("nfft", [16, 32])
+@pytest.mark.parametrize("npol", [1, 2])
+def test_staged_transforms(nfft, npol):
+    rng = np.random.default_rng(nfft + npol)
+    for blocks in (1, 127, 128, 129, 300):
+        n = nfft * blocks + 2
+        v = (rng.standard_normal((npol, 3, n)) + 1j * rng.standard_normal((npol, 3, n))).astype(np.complex64)
+        out = torch.full((3 * nfft, blocks + 1), -1.0, device="cuda")
+        dd.dd_channelise(torch.from_numpy(v.view(np.float32)).cuda(), npol, 3, n, nfft, out, blocks + 1)
+        got = out.cpu().numpy().astype(np.float64)
+        ref = oracle.channelise_power(v, nfft)
+        # float32 transform of log2(nfft) stages: each output within 1e-6 of the largest power, as the other lengths' test
+        assert np.max(np.abs(got[:, :blocks] - ref)) <= 1e-6 * nfft * ref.max()
+        assert np.all(got[:, blocks] == -1.0)
