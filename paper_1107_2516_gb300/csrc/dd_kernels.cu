@@ -335,7 +335,16 @@ row_stats_kernel(const void *__restrict__ out_, int64_t nout, const int32_t *__r
     if constexpr (kInt) {
         const int32_t *x = reinterpret_cast<const int32_t *>(out_) + (size_t)row * nout;
         long long n = 0, s = 0, q = 0;
-        for (int64_t t = tid; t < nout; t += kRowThreads) {
+        int64_t t = tid;
+        for (; t + 7 * kRowThreads < nout; t += 8 * kRowThreads) {     // 8 loads in flight
+            int32_t v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = x[t + u * kRowThreads];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) { s += v[u]; q += (long long)v[u] * v[u]; }
+            n += 8;
+        }
+        for (; t < nout; t += kRowThreads) {
             const long long v = x[t];
             n++; s += v; q += v * v;
         }
@@ -368,7 +377,16 @@ row_stats_kernel(const void *__restrict__ out_, int64_t nout, const int32_t *__r
         const float K = tid < nout ? x[tid] : 0.f;
         float s = 0.f, q = 0.f;
         int n = 0;
-        for (int64_t t = tid; t < nout; t += kRowThreads) {
+        int64_t t = tid;
+        for (; t + 7 * kRowThreads < nout; t += 8 * kRowThreads) {     // 8 loads in flight
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = x[t + u * kRowThreads];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) { const float d = v[u] - K; s += d; q += d * d; }
+            n += 8;
+        }
+        for (; t < nout; t += kRowThreads) {
             const float d = x[t] - K;
             s += d; q += d * d; n++;
         }
@@ -406,18 +424,14 @@ row_stats_kernel(const void *__restrict__ out_, int64_t nout, const int32_t *__r
 }
 
 // ---------------------------------------------------------------------------
-// Boxcar threshold search.  Block = one DM row x kSearchTile samples.  Both
+// Boxcar threshold search.  Block = one DM row x a tile of samples.  Both
 // kernels test a whole run of samples per thread by its largest boxcar sum
 // (one max per sample and width, one comparison per run and width); only runs
-// whose largest sum is a hit are gone through again sample by sample.  A hit's
-// S/N, (B_w - w*mu) / (sigma*sqrt(w)) in double, is formed with its record.
+// whose largest sum is a hit are gone through again sample by sample.  Their
+// hits go to a list in shared memory, so that a pulse's hits, which lie in one
+// or two threads' runs, are finished by all threads of the block: the S/N, (B_w
+// - w*mu) / (sigma*sqrt(w)) in double (slow units here), and the record.
 // ---------------------------------------------------------------------------
-constexpr int kSearchThreads = 256;
-constexpr int kSearchPer = 16;
-constexpr int kSearchTile = kSearchThreads * kSearchPer;
-
-__host__ __device__ __forceinline__ int spad(int i) { return i + (i >> 4); }
-
 // S/N and record of one hit into slot pos.
 __device__ __forceinline__ void put_candidate(dd_candidate *cands, int64_t cap, unsigned long long pos, int row, int w,
                                               int width_idx, int64_t t, double value, const SearchParams *prm,
@@ -436,10 +450,18 @@ __device__ __forceinline__ void put_candidate(dd_candidate *cands, int64_t cap, 
 // Any widths: thread = kSearchPer consecutive samples.  For the widths in
 // ascending order it extends B_w at its first sample from the previous
 // width's sum, then slides it along its samples (B_w(t+1) = B_w(t) + x[t+w] -
-// x[t]); its own samples x[t] stay in registers.  The shared tile is padded
-// one word per 16, so that the threads' windows fall in distinct banks; the
-// step over a pad comes at the same sample for every thread (it depends on w
-// alone), so addresses cost no arithmetic per thread.
+// x[t]); its own samples x[t] stay in registers.  17 samples a thread: an odd
+// stride, so that the threads' words fall in distinct banks without padding
+// and every shared address is the thread's base plus a constant or the width
+// (with 16 samples and a pad word after each 16, index arithmetic was most of
+// the kernel's instructions, and each sample and width was compared): 600
+// rows x 253 443 samples, widths 1, 3, 7, 20, 50, 0.70 -> 0.28 ms.
+constexpr int kSearchThreads = 256;
+constexpr int kSearchPer = 17;
+constexpr int kSearchTile = kSearchThreads * kSearchPer;
+constexpr int kHitList = 1024;      // hits a block finishes per round
+static_assert(kMaxWidths <= 64, "a hit's code holds its width in 6 bits");
+
 template <bool kInt>
 __global__ void __launch_bounds__(kSearchThreads)
 search_kernel(const void *__restrict__ out_, int64_t nout,
@@ -452,9 +474,14 @@ search_kernel(const void *__restrict__ out_, int64_t nout,
     extern __shared__ __align__(16) unsigned char sraw[];
     __shared__ int sw[kMaxWidths], sidx[kMaxWidths];
     __shared__ Acc sthr[kMaxWidths];
+    __shared__ Acc hval[kHitList];                  // the block's hits: their sums and
+    __shared__ int hcode[kHitList];                 // sample << 6 | sorted width
+    __shared__ int nlist;
+    __shared__ unsigned long long first;
     T *x = reinterpret_cast<T *>(sraw);
     const int row = blockIdx.y;
     const int64_t t0 = (int64_t)blockIdx.x * kSearchTile;
+    if (threadIdx.x == 0) nlist = 0;
     const int len = kSearchTile + wmax - 1;
     if (threadIdx.x < nw) {
         const int o = wsorted[nw + threadIdx.x];
@@ -467,19 +494,23 @@ search_kernel(const void *__restrict__ out_, int64_t nout,
     const int64_t avail = nout - t0;
     {
         T r[kSearchPer];
+        if (avail >= kSearchTile) {
 #pragma unroll
-        for (int q = 0; q < kSearchPer; ++q) {
-            const int i = q * kSearchThreads + threadIdx.x;
-            r[q] = i < avail ? __ldcs(src + i) : (T)0;
+            for (int q = 0; q < kSearchPer; ++q) r[q] = __ldcs(src + q * kSearchThreads + threadIdx.x);
+        } else {
+#pragma unroll
+            for (int q = 0; q < kSearchPer; ++q) {
+                const int i = q * kSearchThreads + threadIdx.x;
+                r[q] = i < avail ? __ldcs(src + i) : (T)0;
+            }
         }
 #pragma unroll
-        for (int q = 0; q < kSearchPer; ++q) x[spad(q * kSearchThreads + threadIdx.x)] = r[q];
+        for (int q = 0; q < kSearchPer; ++q) x[q * kSearchThreads + threadIdx.x] = r[q];
     }
-    for (int i = kSearchTile + threadIdx.x; i < len; i += kSearchThreads) x[spad(i)] = i < avail ? src[i] : (T)0;
+    for (int i = kSearchTile + threadIdx.x; i < len; i += kSearchThreads) x[i] = i < avail ? src[i] : (T)0;
     __syncthreads();
     const int base = threadIdx.x * kSearchPer;
-    const T *xb = x + spad(base);                  // this thread's samples, then a pad after every 16
-    if (base >= avail) return;
+    const T *xb = x + base;
     T own[kSearchPer];
 #pragma unroll
     for (int i = 0; i < kSearchPer; ++i) own[i] = xb[i];
@@ -487,16 +518,15 @@ search_kernel(const void *__restrict__ out_, int64_t nout,
     int wprev = 0;
     for (int p = 0; p < nw; ++p) {
         const int w = sw[p];
-        for (int j = wprev; j < w; ++j) b0 += (Acc)xb[spad(j)];
+#pragma unroll 4
+        for (int j = wprev; j < w; ++j) b0 += (Acc)xb[j];
         wprev = w;
         const Acc thr = sthr[p];
-        // x[base + w - 1 + i] for i >= 1: a step over the pad at i == pad
-        const T *xw = xb + spad(w - 1);
-        const int pad = kSearchPer - ((w - 1) & (kSearchPer - 1));
+        const T *xw = xb + (w - 1);              // xw[i] = x[base + i - 1 + w], the sample that enters at i
         Acc b = b0, m = b0;
 #pragma unroll
         for (int i = 1; i < kSearchPer; ++i) {
-            b += (Acc)xw[i + (i >= pad ? 1 : 0)] - (Acc)own[i - 1];
+            b += (Acc)xw[i] - (Acc)own[i - 1];
             if constexpr (kInt) m = b > m ? b : m;
             else m = fmaxf(m, b);
         }
@@ -507,9 +537,22 @@ search_kernel(const void *__restrict__ out_, int64_t nout,
         for (int i = 0; i < kSearchPer; ++i) {
             const int64_t t = t0 + base + i;
             if (t + w > nout) break;
-            if (i > 0) b += (Acc)xw[i + (i >= pad ? 1 : 0)] - (Acc)xb[i - 1];
-            if (b > thr) put_candidate(cands, cap, atomicAdd(count, 1ull), row, w, sidx[p], t, (double)b, prm, rp);
+            if (i > 0) b += (Acc)xw[i] - (Acc)xb[i - 1];
+            if (!(b > thr)) continue;
+            // the list, or (full) the slow way
+            const int at = atomicAdd(&nlist, 1);
+            if (at < kHitList) { hval[at] = b; hcode[at] = (base + i) << 6 | p; }
+            else put_candidate(cands, cap, atomicAdd(count, 1ull), row, w, sidx[p], t, (double)b, prm, rp);
         }
+    }
+    __syncthreads();
+    const int n = min(nlist, kHitList);
+    if (n == 0) return;
+    if (threadIdx.x == 0) first = atomicAdd(count, (unsigned long long)n);
+    __syncthreads();
+    for (int q = threadIdx.x; q < n; q += kSearchThreads) {
+        const int p = hcode[q] & 63;
+        put_candidate(cands, cap, first + q, row, sw[p], sidx[p], t0 + (hcode[q] >> 6), (double)hval[q], prm, rp);
     }
 }
 
@@ -532,8 +575,7 @@ search_kernel(const void *__restrict__ out_, int64_t nout,
 // threads' 16-byte window loads then touch all banks evenly.
 constexpr int kPow2Threads = 128;
 constexpr int kPow2Per = 32;
-static_assert(kPow2Threads * kPow2Per == kSearchTile, "both search kernels use the same tiles");
-constexpr int kHitList = 1024;      // hits a block finishes per round
+constexpr int kPow2Tile = kPow2Threads * kPow2Per;
 
 __host__ __device__ __forceinline__ int spad32(int i) { return i + ((i >> 5) << 2); }
 
@@ -587,7 +629,7 @@ search_pow2_kernel(const void *__restrict__ out_, int64_t nout, const int32_t *_
     __shared__ unsigned long long first;
     T *x = reinterpret_cast<T *>(sraw);
     const int row = blockIdx.y;
-    const int64_t t0 = (int64_t)blockIdx.x * kSearchTile;
+    const int64_t t0 = (int64_t)blockIdx.x * kPow2Tile;
     if (threadIdx.x < K) {
         const int o = wsorted[K + threadIdx.x];     // original index of sorted width 2^threadIdx.x
         sidx[threadIdx.x] = o;
@@ -599,7 +641,7 @@ search_pow2_kernel(const void *__restrict__ out_, int64_t nout, const int32_t *_
     const int64_t avail = nout - t0;                // > 0
     {
         T r[kPow2Per];
-        if (avail >= kSearchTile) {
+        if (avail >= kPow2Tile) {
 #pragma unroll
             for (int q = 0; q < kPow2Per; ++q) r[q] = __ldcs(src + q * kPow2Threads + threadIdx.x);
         } else {
@@ -609,7 +651,7 @@ search_pow2_kernel(const void *__restrict__ out_, int64_t nout, const int32_t *_
                 r[q] = i < avail ? __ldcs(src + i) : (T)0;
             }
         }
-        const int i = kSearchTile + threadIdx.x;
+        const int i = kPow2Tile + threadIdx.x;
         if ((int)threadIdx.x < W) x[spad32(i)] = i < avail ? src[i] : (T)0;
 #pragma unroll
         for (int q = 0; q < kPow2Per; ++q) x[spad32(q * kPow2Threads + threadIdx.x)] = r[q];
@@ -654,9 +696,7 @@ search_pow2_kernel(const void *__restrict__ out_, int64_t nout, const int32_t *_
     }
     if (!__syncthreads_or(hit)) return;
 
-    // Runs with a hit again, sample by sample; their hits through the list, so
-    // that a pulse's hits, which lie in one or two runs, are finished by all
-    // threads of the block.
+    // Runs with a hit again, sample by sample; their hits through the list.
     unsigned hits[K];
 #pragma unroll
     for (int p = 0; p < K; ++p) hits[p] = 0u;
@@ -714,7 +754,7 @@ search_pow2_kernel(const void *__restrict__ out_, int64_t nout, const int32_t *_
 template <bool kInt, int K>
 static void launch_search_pow2(dim3 grid, cudaStream_t s, const void *out, const dd_plan *p)
 {
-    const size_t smem = (size_t)spad32(kSearchTile + kPow2Per + (1 << (K - 1)) + 4) * 4;
+    const size_t smem = (size_t)spad32(kPow2Tile + kPow2Per + (1 << (K - 1)) + 4) * 4;
     search_pow2_kernel<kInt, K><<<grid, kPow2Threads, smem, s>>>(out, p->nsamp_out, p->d_wsorted, p->d_params,
                                                                     p->row_stats ? p->d_rowprm : nullptr,
                                                                     p->d_cands, p->cand_cap, p->d_count);
@@ -981,10 +1021,10 @@ int search_launch(dd_plan *p, const void *out, cudaStream_t s)
     }
     int wmax = 0;
     for (int w : p->widths) wmax = std::max(wmax, w);
-    const int64_t ntile = (p->nsamp_out + kSearchTile - 1) / kSearchTile;
-    dim3 grid((unsigned)ntile, (unsigned)p->ndm);
-    const size_t smem = (size_t)(spad(kSearchTile + wmax - 1) + 1) * 4;
     const int K = pow2_widths(p);
+    const int tile = K ? kPow2Tile : kSearchTile;
+    const dim3 grid((unsigned)((p->nsamp_out + tile - 1) / tile), (unsigned)p->ndm);
+    const size_t smem = (size_t)(kSearchTile + wmax - 1) * 4;
     if (K) {
         if (isint) launch_search_pow2_k<true>(K, grid, s, out, p);
         else launch_search_pow2_k<false>(K, grid, s, out, p);
