@@ -172,7 +172,8 @@ DD_API int dd_last_row_stats(const dd_plan *plan, double *mu_rows, double *sigma
  * and dd_search, and returns the candidates as dd_search does.  With
  * kernels 3 and 5 the copy goes in 8 column chunks on a stream of the plan,
  * and the output tiles each chunk completes are de-dispersed while the next
- * chunk is in flight (same results as the unsplit call).  The plan allocates
+ * chunk is in flight (same results as the unsplit call; a launch of few
+ * blocks is not split).  The plan allocates
  * its device staging for `in` and `out` on the first call and keeps it until
  * dd_plan_destroy.  Synchronises `stream`. */
 DD_API int dd_process_host(dd_plan *plan, const void *in_host, int64_t in_pitch,
@@ -183,7 +184,9 @@ DD_API int dd_process_host(dd_plan *plan, const void *in_host, int64_t in_pitch,
  * first available of tile configurations 12, 11, 9, 10, 5, 3, 6, 4, 1, 0, 2 —
  * kernel 5 shapes where their tables fit the plan, then kernel 3 and kernel 2
  * shapes, in the order of measured speed — or the autotuner's choice;
- * kernel 1 if no tiled configuration fits),
+ * kernel 1 if no tiled configuration fits; a launch that would leave SMs
+ * without a block runs a finer shape of kernel 3, with the same sums, unless
+ * the caller chose a kernel or configuration),
  * 1 = generic shared-memory kernel, 2 = register-blocked kernel (window
  * reused across 4 DM trials per thread), 3 = lane-interleaved kernel (one
  * conflict-free shared load per add, no branches), 4 = tensor-memory window

@@ -288,7 +288,7 @@ int dd_plan_info(const dd_plan *plan, int64_t *maxshift, int64_t *nsamp_out, int
 int dd_plan_set_kernel(dd_plan *plan, int32_t kernel)
 {
     if (!plan) return set_error(DD_ERR_ARG, "plan is NULL");
-    if (kernel == 0) { plan->kernel = plan->fast ? 2 : 1; plan->kernel_req = 0; return DD_OK; }
+    if (kernel == 0) { plan->kernel = plan->fast ? 2 : 1; plan->kernel_req = 0; fast_unforce(plan); return DD_OK; }
     if (kernel == 1) { plan->kernel = 1; plan->kernel_req = 1; return DD_OK; }
     if (kernel == 2) {
         if (!plan->fast) return set_error(DD_ERR_ARG, "kernel 2 is not available for this plan");

@@ -73,6 +73,8 @@ constexpr int kHostChunks = 8;   // input column chunks of the pipelined host pa
 struct FastPlan {
     FastCfgData cfg[kNumFastCfg];
     LaneCfgData lane[kNumLaneCfg];
+    LaneCfgData small;           // kLaneSmall, built for plans whose default launch leaves SMs empty
+    bool forced = false;         // the caller chose the shape: small launches run it too
     TmemCfgData tm[kNumTmemCfg];
     ShareCfgData sh[kNumShareCfg];
     int active = -1;
@@ -133,8 +135,9 @@ static void free_lane(LaneCfgData &c)
 }
 
 // Kernel 3 tables: per (DM block, channel) the aligned row start and every
-// DM trial's offset in the row.  c.ok stays false if rows do not fit.
-static int build_lane(const dd_plan *p, int ti, int dr, int nw, int minb, LaneCfgData &c)
+// DM trial's offset in the row.  c.ok stays false if rows do not fit.  fours:
+// a stage holds a multiple of four channels.
+static int build_lane(const dd_plan *p, int ti, int dr, int nw, int minb, LaneCfgData &c, bool fours = false)
 {
     c = LaneCfgData();
     c.ti = ti; c.dr = dr; c.nw = nw;
@@ -161,7 +164,8 @@ static int build_lane(const dd_plan *p, int ti, int dr, int nw, int minb, LaneCf
     // shared memory of one block: the SM's 228 KB split between `minb` resident blocks
     const size_t budget = std::min<size_t>(p->smem_optin, (228 * 1024) / (size_t)minb - 1024) - 1024;
     const size_t per_ch = (size_t)rs * eb + DB * sizeof(int32_t);
-    const int ch = (int)std::min<size_t>(16, budget / (kStages * per_ch));
+    int ch = (int)std::min<size_t>(16, budget / (kStages * per_ch));
+    if (fours) ch = ch / 4 * 4;
     if (ch < 1) return DD_OK;
     c.bar_off = (int)(((size_t)kStages * ch * per_ch + 15) / 16 * 16);
     c.smem = (size_t)c.bar_off + kStages * sizeof(uint64_t);
@@ -390,10 +394,8 @@ static void share_tables_db(const int32_t *delays, int D, int C, double foff, dd
             }
             prow[np] = rows;
             // stage-1 split: warp w's first row and the pattern holding it.
-            // Warp 0 gets w0 percent of another warp's share of the rows (in
-            // the one-barrier shapes its first thread issues the input copies
-            // and waits while the copy engine takes them), the others equal
-            // shares; packed sums: split_rows.
+            // Warp 0 gets w0 percent of another warp's share of the rows, the
+            // others equal shares; packed sums: split_rows.
             if (kQuad) {
                 nrow.resize(np);
                 for (int q = 0; q < np; ++q) nrow[q] = prow[q + 1] - prow[q];
@@ -433,9 +435,9 @@ static void share_tables_db(const int32_t *delays, int D, int C, double foff, dd
     T.ok = true;
 }
 
-static void share_tables(const int32_t *delays, int D, int C, double foff, dd_dtype dtype, int k, ShareTables &T)
+static void share_tables(const int32_t *delays, int D, int C, double foff, dd_dtype dtype, int k, ShareTables &T,
+                         int w0 = 100)
 {
-    const int w0 = kShareCfg[k].w0;
     switch (kShareCfg[k].dr * kShareCfg[k].nw) {
     case 32: share_tables_db<32>(delays, D, C, foff, dtype, k, T, w0); break;
     case 48: share_tables_db<48>(delays, D, C, foff, dtype, k, T, w0); break;
@@ -685,6 +687,50 @@ static bool cfg_ok(const FastPlan *f, int k)
     return k < kShareBeg ? f->tm[k - kLaneEnd].ok : f->sh[k - kShareBeg].ok;
 }
 
+// The default: the first available configuration in the order of measured
+// speed (kernel 5 shapes where their tables fit, then kernel 3, then kernel 2);
+// the autotuner may change it.
+static int first_cfg(const FastPlan *f)
+{
+    static const int pref[] = {kShareBeg + 3, kShareBeg + 2, kShareBeg + 0, kShareBeg + 1, kNumFastCfg + 2,
+                               kNumFastCfg + 0, kNumFastCfg + 3, kNumFastCfg + 1, 1, 0, 2};
+    for (int k : pref)
+        if (cfg_ok(f, k)) return k;
+    return -1;
+}
+
+// Whether the active shape's launch would leave SMs without a block and the
+// finer shape kLaneSmall, with 8 or 16 times the blocks, is faster.  A block
+// alone on an SM is a chain of loads and adds over all channels.
+// Kernel 3 shapes: 64 trials x 6600 samples of 128 channels (26 blocks) 58 us,
+// 20 us with the finer shape; from one block per SM on the larger shapes'
+// fewer staged samples per sum count for more (512 blocks: 162 against 157 us).
+// Kernel 5 adds fewer words, so there the time decides: measured, one wave of
+// the warp-specialised shape takes 2300 clocks per subband (uint8 1650, of 8
+// channels 1.25 times that), the finer shape 157 per channel or 1.25 per 32
+// words and SM.  1024 channels, 64 trials x 8192 samples: 298 -> 113 us (uint8
+// 214 -> 87); 128 x 16384: 307 and 287 (216 and 234).
+static bool few_blocks(const dd_plan *p, const FastPlan *f)
+{
+    const int k = f->active;
+    auto blocks = [&](int ti, int db) {
+        return ((p->nsamp_out + 32 * ti - 1) / (32 * ti)) * (int64_t)((p->ndm + db - 1) / db);
+    };
+    if (k >= kNumFastCfg && k < kLaneEnd) {
+        const LaneShape &l = kLaneCfg[k - kNumFastCfg];
+        return blocks(l.ti, l.dr * l.nw) < p->sm_count;
+    }
+    if (k < kShareBeg) return false;
+    const ShareShape &sh = kShareCfg[k - kShareBeg];
+    const ShareCfgData &c = f->sh[k - kShareBeg];
+    // float sums of 8-channel subbands are rounded in another order: not to the bit
+    if (p->nchans % 4 || (c.cs == 8 && p->dtype != DD_U8) || blocks(sh.ti, sh.dr * sh.nw) > p->sm_count) return false;
+    const double wave = c.nsub * (p->dtype == DD_U8 ? 1650.0 : 2300.0) * (c.cs == 8 ? 1.25 : 1.0);
+    const int db = kLaneSmall.dr * kLaneSmall.nw, tile = 32 * kLaneSmall.ti;
+    const double words = (double)blocks(kLaneSmall.ti, db) * db * tile * p->nchans / 32;
+    return std::max(157.0 * p->nchans, 1.25 * words / p->sm_count) < wave;
+}
+
 int fast_configure(dd_plan *p)
 {
     p->fast = nullptr;
@@ -698,11 +744,15 @@ int fast_configure(dd_plan *p)
     for (int k = 0; k < kNumTmemCfg && rc == DD_OK; ++k)
         rc = build_tmem(p, kTmemCfg[k].n, kTmemCfg[k].dbw, kTmemCfg[k].nw, f->tm[k]);
     for (int k = 0; k < kNumShareCfg && rc == DD_OK; ++k) rc = build_share(p, k, f->sh[k]);
+    // the finer shape only for plans whose default launch it would replace
+    if (rc == DD_OK && (f->active = first_cfg(f)) >= 0 && few_blocks(p, f))
+        rc = build_lane(p, kLaneSmall.ti, kLaneSmall.dr, kLaneSmall.nw, kLaneSmall.minb, f->small, true);
     cudaError_t e = cudaSuccess;
     for (int k = 0; k < kNumFastCfg && rc == DD_OK && e == cudaSuccess; ++k)
         if (f->cfg[k].ok) e = prepare_cfg(k, p->smem_optin);
     for (int k = 0; k < kNumLaneCfg && rc == DD_OK && e == cudaSuccess; ++k)
         if (f->lane[k].ok) e = prepare_lane(k, p->smem_optin);
+    if (rc == DD_OK && e == cudaSuccess && f->small.ok) e = lane_prepare_small(p->smem_optin);
     for (int k = 0; k < kNumTmemCfg && rc == DD_OK && e == cudaSuccess; ++k)
         if (f->tm[k].ok) e = prepare_tmem(k, p->smem_optin);
     for (int k = 0; k < kNumShareCfg && rc == DD_OK && e == cudaSuccess; ++k)
@@ -712,13 +762,6 @@ int fast_configure(dd_plan *p)
     p->fast = f;
     if (rc == DD_OK && e != cudaSuccess) rc = cuda_fail(e, "kernel 2 setup");
     if (rc != DD_OK) { fast_release(p); return rc; }
-    // default: the first available configuration in the order of measured
-    // speed (kernel 5 shapes where their tables fit, then kernel 3, then
-    // kernel 2); the autotuner may change it
-    static const int pref[] = {kShareBeg + 3, kShareBeg + 2, kShareBeg + 0, kShareBeg + 1, kNumFastCfg + 2,
-                               kNumFastCfg + 0, kNumFastCfg + 3, kNumFastCfg + 1, 1, 0, 2};
-    for (int k : pref)
-        if (cfg_ok(f, k)) { f->active = k; break; }
     if (f->active < 0) { fast_release(p); return DD_OK; }   // tiled kernels unavailable
     std::lock_guard<std::mutex> g(g_tune_mu);
     auto it = g_tune_cache.find(tune_key(p));
@@ -753,7 +796,8 @@ static int lane_run(dd_plan *p, int k, int dgroup, const void *in, int64_t pitch
                     int64_t tile_lo = 0, int64_t tile_hi = -1)
 {
     FastPlan *f = static_cast<FastPlan *>(p->fast);
-    LaneCfgData &c = f->lane[k];
+    const bool small = k < 0;    // kLaneSmall, in kernel 5's order if that is the plan's kernel
+    LaneCfgData &c = small ? f->small : f->lane[k];
     const int tile = 32 * c.ti;
     const int64_t ntile = (p->nsamp_out + tile - 1) / tile;
     if (ntile * c.nblk > INT32_MAX) return generic_execute(p, in, pitch, out, s);
@@ -772,7 +816,7 @@ static int lane_run(dd_plan *p, int k, int dgroup, const void *in, int64_t pitch
     a.dgroup = std::max(1, std::min(dgroup, c.nblk));
     a.out = out; a.err = f->d_err; a.smem = c.smem;
     a.partials = static_cast<char *>(p->d_partials) + (size_t)(tile_lo * c.nblk) * stat_bytes(p);
-    cudaError_t e = launch_lane(k, p->dtype, a, s);
+    cudaError_t e = small ? lane_launch_small(p->dtype, a, f->active >= kShareBeg, s) : launch_lane(k, p->dtype, a, s);
     if (e != cudaSuccess) return cuda_fail(e, "launch lane_kernel");
     p->n_partials = np;
     p->stats_out = out;
@@ -893,6 +937,7 @@ int fast_execute(dd_plan *p, const void *in, int64_t pitch, void *out, cudaStrea
             return generic_execute(p, in, pitch, out, s);
         return fast_run(p, k, f->dgroup, in, pitch, out, s);
     }
+    if (f->small.ok && !f->forced && few_blocks(p, f)) return lane_run(p, -1, f->dgroup, in, pitch, out, s);
     return fast_run(p, f->active, f->dgroup, in, pitch, out, s);
 }
 
@@ -926,6 +971,7 @@ int fast_execute_host(dd_plan *p, const void *in_host, int64_t pitch, void *in_d
 {
     FastPlan *f = static_cast<FastPlan *>(p->fast);
     if (!f || ((uintptr_t)in_dev & 15u) || (pitch % f->al)) return kNotPipelined;
+    if (f->small.ok && !f->forced && few_blocks(p, f)) return kNotPipelined;   // one small launch
     const int k = f->active;
     int tile, nblk;
     int64_t reach;
@@ -1035,7 +1081,13 @@ int fast_set_tile(dd_plan *p, int cfg, int dgroup)
     if (dgroup < 1) return set_error(DD_ERR_ARG, "raster group must be >= 1");
     f->active = cfg;
     f->dgroup = dgroup;
+    f->forced = true;
     return DD_OK;
+}
+
+void fast_unforce(dd_plan *p)
+{
+    if (p->fast) static_cast<FastPlan *>(p->fast)->forced = false;
 }
 
 int fast_get_tile(const dd_plan *p, int *cfg, int *dgroup, int *tr, int *nw)
@@ -1074,9 +1126,10 @@ void fast_release(dd_plan *p)
     if (!f) return;
     for (int k = 0; k < kNumFastCfg; ++k) free_cfg(f->cfg[k]);
     for (int k = 0; k < kNumLaneCfg; ++k) free_lane(f->lane[k]);
+    free_lane(f->small);
+    if (f->d_err) cudaFree(f->d_err);
     for (int k = 0; k < kNumTmemCfg; ++k) free_tmem(f->tm[k]);
     for (int k = 0; k < kNumShareCfg; ++k) free_share(f->sh[k]);
-    if (f->d_err) cudaFree(f->d_err);
     if (f->copy_stream) {
         cudaStreamSynchronize(f->copy_stream);
         for (int i = 0; i <= kHostChunks; ++i)
@@ -1397,7 +1450,7 @@ int dd_share_tables(const int32_t *delays, int32_t ndm, int32_t nchans, double f
     if (config < kShareBeg || config >= kShareBeg + kNumShareCfg)
         return set_error(DD_ERR_ARG, "configuration %d is not a kernel 5 shape", config);
     ShareTables T;
-    share_tables(delays, ndm, nchans, foff, (dd_dtype)dtype, config - kShareBeg, T);
+    share_tables(delays, ndm, nchans, foff, (dd_dtype)dtype, config - kShareBeg, T, kShareCfg[config - kShareBeg].w0);
     info[0] = T.ok ? 1 : 0;
     info[1] = T.nblk; info[2] = T.nsub; info[3] = T.rs; info[4] = T.pmax; info[5] = T.klen;
     if (!T.ok) return DD_OK;

@@ -153,5 +153,6 @@ int fast_autotune(dd_plan *p, const void *in, int64_t pitch, void *out, cudaStre
 int fast_set_tile(dd_plan *p, int cfg, int dgroup);
 int fast_get_tile(const dd_plan *p, int *cfg, int *dgroup, int *tr, int *nw);
 int fast_kernel_id(const dd_plan *p);
+void fast_unforce(dd_plan *p);     // the active shape counts as the default again
 
 }  // namespace dd

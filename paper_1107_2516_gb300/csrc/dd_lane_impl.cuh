@@ -137,7 +137,10 @@ __device__ __forceinline__ void lane_raster(const LaneLaunch &a, int64_t lin, in
 // symbol (not a pointer argument), so that its loads and stores stay
 // shared-space instructions in the out-of-line copies the persistent kernels
 // call.
-template <typename Tin, bool kInt, int TI, int DR, int NW>
+// kFours (ch a multiple of 4, nchans too): four channels are summed before
+// they are added, kernel 5's order with subbands of 4 and so its float sums to
+// the bit.
+template <typename Tin, bool kInt, int TI, int DR, int NW, bool kFours = false>
 __device__ __forceinline__ bool lane_tile(const LaneLaunch &a, int blk, int64_t t0, int64_t lin,
                                           uint64_t *bar, uint32_t &gstage)
 {
@@ -212,6 +215,27 @@ __device__ __forceinline__ bool lane_tile(const LaneLaunch &a, int blk, int64_t 
         const Tin *srow = rows + (size_t)buf * stage_elems + lane;
         const int32_t *so = soffs + (size_t)buf * ch * kDmBlk + warp * DR;
         if constexpr (kBytes) bs.add_stage(srow - lane, rs, so, kDmBlk, cn, lane);
+        else if constexpr (kFours) for (int cc = 0; cc < cn; cc += 4) {
+            const Tin *r = srow + (size_t)cc * rs;
+#pragma unroll
+            for (int j = 0; j < DR; j += 4) {
+                int o[4][4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const int4 v = *reinterpret_cast<const int4 *>(so + (cc + c) * kDmBlk + j);
+                    o[0][c] = v.x; o[1][c] = v.y; o[2][c] = v.z; o[3][c] = v.w;
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+#pragma unroll
+                    for (int i = 0; i < TI; ++i) {
+                        float v = lane_ld<Tin>(r + o[e][0] + 32 * i);
+#pragma unroll
+                        for (int c = 1; c < 4; ++c) v += lane_ld<Tin>(r + c * rs + o[e][c] + 32 * i);
+                        acc[j + e][i] += v;
+                    }
+            }
+        }
         else for (int cc = 0; cc < cn; ++cc) {
             const Tin *r = srow + (size_t)cc * rs;
             // the warp's DR offsets: uniform 16-byte loads, one shared-memory
@@ -289,7 +313,7 @@ __device__ __forceinline__ bool lane_tile(const LaneLaunch &a, int blk, int64_t 
 }
 
 // One plan: one block per work item, grid = nblk * ntile.
-template <typename Tin, bool kInt, int TI, int DR, int NW, int MINB>
+template <typename Tin, bool kInt, int TI, int DR, int NW, int MINB, bool kFours = false>
 __global__ void __launch_bounds__(NW * 32, MINB) lane_kernel(LaneLaunch a)
 {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -304,7 +328,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) lane_kernel(LaneLaunch a)
     lane_raster<TI>(a, blockIdx.x, blk, t0);
     t0 += a.t_base;
     uint32_t gstage = 0;
-    lane_tile<Tin, kInt, TI, DR, NW>(a, blk, t0, blockIdx.x, bar, gstage);
+    lane_tile<Tin, kInt, TI, DR, NW, kFours>(a, blk, t0, blockIdx.x, bar, gstage);
 }
 
 // lane_tile as an out-of-line function: the persistent kernel calls one per
@@ -365,26 +389,33 @@ __global__ void __launch_bounds__(NW * 32, MINB) lane_batch_kernel(LaneBatchLaun
     }
 }
 
-template <int TI, int DR, int NW, int MINB>
+template <int TI, int DR, int NW, int MINB, bool kFours = false>
 cudaError_t lane_launch_cfg(dd_dtype t, const LaneLaunch &a, cudaStream_t s)
 {
     const unsigned grid = (unsigned)(a.ntile * a.nblk);
     switch (t) {
-    case DD_F32: lane_kernel<float, false, TI, DR, NW, MINB><<<grid, NW * 32, a.smem, s>>>(a); break;
-    case DD_F16: lane_kernel<__half, false, TI, DR, NW, MINB><<<grid, NW * 32, a.smem, s>>>(a); break;
+    case DD_F32: lane_kernel<float, false, TI, DR, NW, MINB, kFours><<<grid, NW * 32, a.smem, s>>>(a); break;
+    case DD_F16: lane_kernel<__half, false, TI, DR, NW, MINB, kFours><<<grid, NW * 32, a.smem, s>>>(a); break;
     case DD_U8: lane_kernel<uint8_t, true, TI, DR, NW, MINB><<<grid, NW * 32, a.smem, s>>>(a); break;
     }
     return cudaGetLastError();
 }
 
+template <int TI, int DR, int NW, int MINB, bool kFours = false>
+cudaError_t lane_prepare_one(size_t optin)
+{
+    cudaError_t e = allow_max_dynamic_smem((const void *)lane_kernel<float, false, TI, DR, NW, MINB, kFours>, optin);
+    if (e == cudaSuccess)
+        e = allow_max_dynamic_smem((const void *)lane_kernel<__half, false, TI, DR, NW, MINB, kFours>, optin);
+    if (e == cudaSuccess)
+        e = allow_max_dynamic_smem((const void *)lane_kernel<uint8_t, true, TI, DR, NW, MINB>, optin);
+    return e;
+}
+
 template <int TI, int DR, int NW, int MINB>
 cudaError_t lane_prepare_cfg(size_t optin)
 {
-    cudaError_t e = allow_max_dynamic_smem((const void *)lane_kernel<float, false, TI, DR, NW, MINB>, optin);
-    if (e == cudaSuccess)
-        e = allow_max_dynamic_smem((const void *)lane_kernel<__half, false, TI, DR, NW, MINB>, optin);
-    if (e == cudaSuccess)
-        e = allow_max_dynamic_smem((const void *)lane_kernel<uint8_t, true, TI, DR, NW, MINB>, optin);
+    cudaError_t e = lane_prepare_one<TI, DR, NW, MINB>(optin);
     if (e == cudaSuccess)
         e = allow_max_dynamic_smem((const void *)lane_batch_kernel<TI, DR, NW, MINB>, optin);
     return e;
@@ -404,6 +435,13 @@ cudaError_t lane_batch_launch_cfg(const LaneBatchLaunch &b, int sms, size_t smem
 struct LaneShape { int ti, dr, nw, minb; };
 constexpr int kNumLaneCfg = 4;
 constexpr LaneShape kLaneCfg[kNumLaneCfg] = {{16, 4, 8, 2}, {16, 8, 8, 1}, {16, 8, 4, 3}, {8, 16, 4, 3}};
+
+// A finer shape for launches whose blocks would not fill the SMs (16 trials x
+// 128 samples a block instead of 32 x 512 or kernel 5's 64 x 512): the same
+// sums in kernel 3's order or (fours) in kernel 5's.
+constexpr LaneShape kLaneSmall = {4, 4, 4, 4};
+cudaError_t lane_launch_small(dd_dtype t, const LaneLaunch &a, bool fours, cudaStream_t s);
+cudaError_t lane_prepare_small(size_t optin);
 
 cudaError_t lane_launch_c0(dd_dtype t, const LaneLaunch &a, cudaStream_t s);
 cudaError_t lane_launch_c1(dd_dtype t, const LaneLaunch &a, cudaStream_t s);

@@ -319,8 +319,9 @@ int dd_server_add_beam(dd_server *S, int32_t nchans, double fch1, double foff, d
             } else {
                 rc = cuda_fail(e, "admission stream");
             }
-        } else if (dd_plan_set_kernel(b->plan, 5) != DD_OK) {
-            set_error(DD_OK, "%s", "");
+        } else {
+            if (dd_plan_set_kernel(b->plan, 5) != DD_OK) set_error(DD_OK, "%s", "");
+            fast_unforce(b->plan);     // short chunks may take the finer shape
         }
     }
     std::lock_guard<std::mutex> g(S->mu);

@@ -369,7 +369,8 @@ __device__ __forceinline__ void share_stat_flush(const ShareLaunch &a, const Sha
 // One work item: DM block `blk` x the time tile at t0; partial statistics
 // record `lin`.  bar[NS] is the block's input ring; `gstage` its running stage
 // count (a persistent block keeps the ring across items: subband s of this
-// item uses buffer (gstage + s) % NS, parity ((gstage + s) / NS) & 1).
+// item uses buffer (gstage + s) % NS, parity ((gstage + s) / NS) & 1; each
+// warp arrives once per stage).
 // Returns false if a bounded wait gave up.
 template <typename Tin, bool kInt, int TI, int DR, int NW, int CS, int NPMAX, int NS>
 __device__ __forceinline__ bool share_tile(const ShareLaunch &a, int blk, int64_t t0, int64_t lin,
@@ -389,43 +390,33 @@ __device__ __forceinline__ bool share_tile(const ShareLaunch &a, int blk, int64_
     int32_t *srec = reinterpret_cast<int32_t *>(smem + NS * stage_elems * sizeof(Tin));
     float *P = reinterpret_cast<float *>(srec + NS * R::kLen);
     const int32_t *brec = a.rec + (size_t)blk * nsub * R::kLen;
-    const int32_t *bbase = a.base + (size_t)blk * a.nchans;
     const uint32_t g0 = gstage;
     gstage += (uint32_t)nsub;
 
-    // thread 0 issues subband s's copies with its rows' start offsets loaded
-    // one subband earlier (the global loads' latency stays off the barrier path)
-    // each channel's row: the rl elements its DM trials read from column
-    // t0 + b on (fewer than rs near the top of the band), cut at the input's end
-    auto row_bytes = [&](int b, int rl, int64_t &g) -> uint32_t {
-        g = t0 + b;
-        int64_t n = a.nsamp_in_al - g;
-        n = n < 0 ? 0 : (n > rl ? rl : n);
-        return (uint32_t)(n * (int64_t)sizeof(Tin));
-    };
-    auto issue = [&](int s, const int (&rb)[CS], const int (&rl)[CS]) {
-        const int buf = (int)((g0 + s) % NS);
-        uint32_t bytes = (uint32_t)(R::kLen * sizeof(int32_t));
-#pragma unroll
-        for (int cc = 0; cc < CS; ++cc) { int64_t g; bytes += row_bytes(rb[cc], rl[cc], g); }
-        mbar_arrive_tx(&bar[buf], bytes);
-        bulk_g2s(srec + (size_t)buf * R::kLen, brec + (size_t)s * R::kLen, (uint32_t)(R::kLen * sizeof(int32_t)),
-                 &bar[buf]);
-        const uint64_t pol = l2_evict_last();          // other DM blocks of this tile stage these rows soon
-#pragma unroll
-        for (int cc = 0; cc < CS; ++cc) {
-            int64_t g;
-            const uint32_t nb = row_bytes(rb[cc], rl[cc], g);
-            if (nb)
-                bulk_g2s_hint(rows + (size_t)buf * stage_elems + (size_t)cc * rs,
-                              in + (size_t)(s * CS + cc) * a.pitch + g, nb, &bar[buf], pol);
-        }
-    };
-    const int32_t *blen = a.rlen + (size_t)blk * a.nchans;
-    int rb[CS], rl[CS];
+    // Warp w < CS issues row w of subband s, the last warp the record: a bulk
+    // copy holds the thread that issues it some 270 cycles, so they are spread.
+    // A row's start and length are loaded one subband early (the global loads'
+    // latency stays off the barrier path); the row is the rl elements that
+    // the block's DM trials read from column t0 + b on, cut at the input's end.
+    static_assert(CS <= NW, "a warp per row");
+    int rb = 0, rl = 0;                                // of the next subband to issue
     auto load_rb = [&](int s) {
-#pragma unroll
-        for (int cc = 0; cc < CS; ++cc) { rb[cc] = bbase[s * CS + cc]; rl[cc] = blen[s * CS + cc]; }
+        const size_t i = (size_t)blk * a.nchans + s * CS + min(warp, CS - 1);
+        rb = a.base[i];
+        rl = a.rlen[i];
+    };
+    auto issue = [&](int s) {
+        if (lane != 0) return;
+        const int buf = (int)((g0 + s) % NS);
+        const int64_t g = t0 + rb;
+        int64_t n = a.nsamp_in_al - g;
+        n = n < 0 || warp >= CS ? 0 : (n > rl ? rl : n);
+        const uint32_t nb = (uint32_t)(n * (int64_t)sizeof(Tin)), rec_b = (uint32_t)(R::kLen * sizeof(int32_t));
+        mbar_arrive_tx(&bar[buf], nb + (warp == NW - 1 ? rec_b : 0u));
+        if (warp == NW - 1) bulk_g2s(srec + (size_t)buf * R::kLen, brec + (size_t)s * R::kLen, rec_b, &bar[buf]);
+        if (nb)
+            bulk_g2s_hint(rows + (size_t)buf * stage_elems + (size_t)warp * rs, in + (size_t)(s * CS + warp) * a.pitch + g,
+                          nb, &bar[buf], l2_evict_last());   // other DM blocks of this tile stage these rows soon
     };
 
     float acc[DR][TI];
@@ -434,16 +425,14 @@ __device__ __forceinline__ bool share_tile(const ShareLaunch &a, int blk, int64_
 #pragma unroll
         for (int i = 0; i < TI; ++i) acc[j][i] = 0.f;
 
-    if (tid == 0) {
-        for (int s = 0; s < NS - 1 && s < nsub; ++s) { load_rb(s); issue(s, rb, rl); }
-        if (NS - 1 < nsub) load_rb(NS - 1);
-    }
+    for (int s = 0; s < NS - 1 && s < nsub; ++s) { load_rb(s); issue(s); }
+    if (NS - 1 < nsub) load_rb(NS - 1);
 
     bool ok = true;
     int q[DR];
     for (int s = 0; s < nsub; ++s) {
-        if (tid == 0 && s + NS - 1 < nsub) {
-            issue(s + NS - 1, rb, rl);
+        if (s + NS - 1 < nsub) {
+            issue(s + NS - 1);
             if (s + NS < nsub) load_rb(s + NS);
         }
         const int buf = (int)((g0 + s) % NS);
@@ -484,7 +473,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) share_kernel(ShareLaunch a)
     extern __shared__ __align__(128) unsigned char smem[];
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + a.bar_off);
     if (threadIdx.x == 0) {
-        for (int s = 0; s < NS; ++s) mbar_init(&bar[s], 1);
+        for (int s = 0; s < NS; ++s) mbar_init(&bar[s], NW);
         mbar_fence_init();
     }
     __syncthreads();
@@ -517,7 +506,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) mixed_batch_kernel(LaneBatchLau
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + b.bar_off), *sbar = bar + kStages;
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) mbar_init(&bar[s], NW);
-        for (int s = 0; s < NS; ++s) mbar_init(&sbar[s], 1);
+        for (int s = 0; s < NS; ++s) mbar_init(&sbar[s], NW);
         mbar_fence_init();
     }
     __syncthreads();
@@ -875,11 +864,9 @@ __global__ void __launch_bounds__((NW + PW + kWsStage) * 32, 1) share_ws_kernel(
 // per SM the register budget targets, input stages (at most, in the
 // warp-specialised form), stage-1 warps (0: the one-barrier-per-subband
 // kernel, whose warps do both stages), partial-sum slots, stage-1 rows of warp
-// 0 in percent of another warp's (its first thread issues the one-barrier
-// kernels' input copies, which hold it for ~1000 cycles per subband: a smaller
-// share keeps it from being the last one at each subband's barrier.  The
-// warp-specialised kernel's split gives every stage-1 warp an equal share;
-// its value here only enters dd_share_tables' records)}.
+// 0 in percent of another warp's in dd_share_tables' records (from the time
+// when its first thread issued all input copies; the kernels' own tables give
+// every warp an equal share)}.
 constexpr int kShCS = 4, kShNP = 16;
 struct ShareShape { int ti, dr, nw, minb, ns, pw, pb, w0; };
 constexpr int kNumShareCfg = 4;

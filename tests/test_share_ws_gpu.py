@@ -59,3 +59,35 @@ def test_largest_bytes():
     x = np.full((nch, nsamp), 255, np.uint8)
     got, mu, _ = run(x, 0, nsamp + 4, d, m, nch, fch1, foff, ts, dms, nsamp, "u8")
     assert np.all(got == 255 * nch) and mu == 255.0 * nch
+
+
+@pytest.mark.parametrize("dtype", ["f32", "u8", "f16"])
+@pytest.mark.parametrize("case", list(range(len(CASES))) + ["kernel 3"])
+def test_launches_of_few_blocks_give_the_same_sums(case, dtype):
+    # the finer shape that a plan left to itself runs, against the shape it stands for
+    if case == "kernel 3":                       # more delay patterns than kernel 5 takes
+        nch, fch1, foff, ts, dms, nsamp, cfg = 128, 150.0, -0.1953125, 327.68e-6, [0.1 * i for i in range(41)], 3000, 5
+    else:
+        (nch, fch1, foff, ts, dms, nsamp, _), cfg = CASES[case], 12
+    al = 16 // {"f32": 4, "u8": 1, "f16": 2}[dtype]
+    x = synth.noise_f32(nch, nsamp, 3)
+    x = synth.quantize_u8(x) if dtype == "u8" else x.astype(np.float16) if dtype == "f16" else x
+    pitch = -(-nsamp // al) * al
+    pad = np.zeros((nch, pitch), x.dtype)
+    pad[:, :nsamp] = x
+    dev = torch.from_numpy(pad.view(np.int16) if dtype == "f16" else pad).cuda()
+    got = []
+    for forced in (False, True):
+        plan = dd.Plan(nch, fch1, foff, ts, dms, [1, 2], 3.0, TYPE[dtype], nsamp)
+        assert plan.kernel == (3 if case == "kernel 3" else 5)
+        if forced:
+            plan.set_tile(cfg, 8)
+        out = torch.full((len(dms) * plan.nsamp_out + 16,), -7, dtype=torch.int32 if dtype == "u8" else torch.float32, device="cuda")
+        plan.execute(dev, pitch, out)
+        cands, total = plan.search(out, capacity=1 << 18)
+        host, n_host = plan.process_host(pad.view(np.int16) if dtype == "f16" else pad, pitch, capacity=1 << 18)
+        assert n_host == total and np.array_equal(host, cands)
+        got.append((out.cpu().numpy(), plan.stats()))
+        plan.close()
+    assert np.array_equal(got[0][0], got[1][0]) and np.all(got[0][0][-16:] == -7)
+    assert got[0][1] == pytest.approx(got[1][1], rel=1e-5, abs=1e-5)
