@@ -757,8 +757,7 @@ int fast_configure(dd_plan *p)
         if (f->tm[k].ok) e = prepare_tmem(k, p->smem_optin);
     for (int k = 0; k < kNumShareCfg && rc == DD_OK && e == cudaSuccess; ++k)
         if (f->sh[k].ok) e = share_prepare(k, p->smem_optin);
-    if (rc == DD_OK && e == cudaSuccess) e = cudaMalloc(&f->d_err, sizeof(int));
-    if (rc == DD_OK && e == cudaSuccess) e = cudaMemset(f->d_err, 0, sizeof(int));
+    f->d_err = &p->d_back->err;
     p->fast = f;
     if (rc == DD_OK && e != cudaSuccess) rc = cuda_fail(e, "kernel 2 setup");
     if (rc != DD_OK) { fast_release(p); return rc; }
@@ -1127,7 +1126,6 @@ void fast_release(dd_plan *p)
     for (int k = 0; k < kNumFastCfg; ++k) free_cfg(f->cfg[k]);
     for (int k = 0; k < kNumLaneCfg; ++k) free_lane(f->lane[k]);
     free_lane(f->small);
-    if (f->d_err) cudaFree(f->d_err);
     for (int k = 0; k < kNumTmemCfg; ++k) free_tmem(f->tm[k]);
     for (int k = 0; k < kNumShareCfg; ++k) free_share(f->sh[k]);
     if (f->copy_stream) {
@@ -1601,11 +1599,13 @@ int dd_batch_results(dd_batch *B, int32_t beam, dd_candidate *cand_host, int64_t
     if (!B || beam < 0 || beam >= (int)B->plans.size()) return set_error(DD_ERR_ARG, "bad beam index");
     if (!n_found || capacity < 0 || (capacity > 0 && !cand_host)) return set_error(DD_ERR_ARG, "bad arguments");
     cudaStream_t s = (cudaStream_t)stream;
-    int h = 0;
-    cudaError_t e = cudaMemcpyAsync(&h, B->d_err, sizeof(int), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return cuda_fail(e, "batch status");
-    if (h) return set_error(h, "batch kernel gave up waiting for its input copies");
+    if (B->cfg >= 0 && B->cfg < kNumFastCfg) {      // kernel 2's grid has one status for all beams
+        int h = 0;
+        cudaError_t e = cudaMemcpyAsync(&h, B->d_err, sizeof(int), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) return cuda_fail(e, "batch status");
+        if (h) return set_error(h, "batch kernel gave up waiting for its input copies");
+    }
     dd_plan *p = B->plans[beam];
     return search_readback(p, cand_host, capacity, n_found, s, p->cand_cap);
 }

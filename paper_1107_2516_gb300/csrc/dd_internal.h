@@ -36,6 +36,15 @@ struct FinScratch {
     unsigned int ticket;
 };
 
+// What the host reads back after a search, in one copy: the statistics and
+// thresholds, the hit count, and the status that a kernel of the plan left.
+struct SearchBack {
+    SearchParams prm;
+    unsigned long long count;
+    int err, pad_;
+};
+constexpr int kBackCands = 512;  // candidates that come with it
+
 constexpr int kMaxWidths = 64;
 
 // Per-DM-row statistics and thresholds (search option: statistics of each DM
@@ -85,14 +94,14 @@ struct dd_plan {
     int64_t n_partials = 0;
     const void *stats_out = nullptr;       // out buffer the partials describe
     // search
-    dd::SearchParams *d_params = nullptr;
+    dd::SearchBack *d_back = nullptr, *h_back = nullptr;   // h_back pinned
+    dd::SearchParams *d_params = nullptr;  // in d_back
     dd::FinScratch *d_fin = nullptr;
     int32_t *d_wsorted = nullptr;          // widths sorted ascending: [nw] widths, [nw] indices
     dd_candidate *d_cands = nullptr;
     int64_t cand_cap = 0;
-    unsigned long long *d_count = nullptr;
-    unsigned long long *h_count = nullptr; // pinned
-    dd::SearchParams *h_params = nullptr;  // pinned
+    unsigned long long *d_count = nullptr; // in d_back
+    dd_candidate *h_cands = nullptr;       // pinned [kBackCands]
     double last_mu = 0, last_sigma = 0;
     // per-DM-row statistics option
     int32_t row_stats = 0;                 // 0: whole buffer (Section 3), 1: per DM row

@@ -336,7 +336,7 @@ struct dd_subband_plan {
     int64_t maxshift = 0, nsamp_out = 0, L = 0;
     SubStage st1, st2;
     float *d_inter = nullptr;         // [nsub][K][L] partially de-dispersed series
-    int *d_err = nullptr;
+    int *d_err = nullptr;             // the fine plan's status, read back with its search
 };
 
 static void free_subband(dd_subband_plan *p)
@@ -345,7 +345,6 @@ static void free_subband(dd_subband_plan *p)
     p->st1.release();
     p->st2.release();
     if (p->d_inter) cudaFree(p->d_inter);
-    if (p->d_err) cudaFree(p->d_err);
     if (p->fine) dd_plan_destroy(p->fine);
     delete p;
 }
@@ -439,8 +438,7 @@ int dd_subband_plan_create(int32_t nchans, double fch1_mhz, double foff_mhz, dou
     if (rc == DD_OK) rc = finish_stage(p->st2, need2, 4, f->smem_optin);
     if (rc) { free_subband(p); return rc; }
     cudaError_t e = sub_prepare(f->smem_optin);
-    if (e == cudaSuccess) e = cudaMalloc(&p->d_err, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(p->d_err, 0, sizeof(int));
+    p->d_err = &f->d_back->err;
     if (e != cudaSuccess) { rc = cuda_fail(e, "subband setup"); free_subband(p); return rc; }
     *plan_out = p;
     return DD_OK;
@@ -529,16 +527,7 @@ int dd_subband_search(dd_subband_plan *plan, const void *out_dev, dd_candidate *
                       int64_t capacity, int64_t *n_found, void *stream)
 {
     if (!plan) return set_error(DD_ERR_ARG, "plan is NULL");
-    const int rc = dd_search(plan->fine, out_dev, cand_host, capacity, n_found, stream);
-    if (rc != DD_OK && rc != DD_ERR_OVERFLOW) return rc;
-    int h = 0;
-    cudaError_t e = cudaMemcpy(&h, plan->d_err, sizeof(int), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(e, "read subband status");
-    if (h) {
-        cudaMemset(plan->d_err, 0, sizeof(int));
-        return set_error(h, "subband kernel gave up waiting for its input copies (status %d)", h);
-    }
-    return rc;
+    return dd_search(plan->fine, out_dev, cand_host, capacity, n_found, stream);
 }
 
 int dd_subband_last_stats(const dd_subband_plan *plan, double *mu, double *sigma)
