@@ -197,8 +197,8 @@ __device__ __forceinline__ void share_stage1(const int32_t *rec, const Tin *srow
 // with one byte load (and a conversion to float) per term; stage 2 reads half
 // the words.  Bound by instructions, no longer by shared memory (ncu: issue
 // 71%, shared-memory wavefronts 60% of their peaks).  LOFAR-like beam of 2^18
-// uint8 samples, 2000 trials: 30.0 -> 20.7 ms; 4096 channels x 65536 samples,
-// 1500 trials: 24.7 -> 14.1 ms.  A single step where one row is left instead of a pair,
+// uint8 samples, 2000 trials: 30.0 -> 20.2 ms; 4096 channels x 65536 samples,
+// 1500 trials: 24.7 -> 13.5 ms.  Exact step sizes for the rows that are left,
 // and the high half added with one dp2a instead of a shift and an add, are
 // 1.10x of that.
 template <typename R, int CS, int NW>
@@ -265,10 +265,16 @@ __device__ __forceinline__ void share_stage1_bytes(const int32_t *rec, const uin
                 }
             }
         };
-        constexpr int kStep = CS == 4 ? 2 : 1;                  // 16 loads a step
-        for (; r + kStep <= rend; r += kStep, g += 32 * kStep) rows(std::integral_constant<int, kStep>());
-        if (r < rend) rows(std::integral_constant<int, 1>());
-        r = rend;
+        // 32 loads a step, then the leftover rows (pairs only: 5% longer)
+        constexpr int kStep = CS == 4 ? 4 : 2;
+        auto step = [&](auto n) {
+            rows(n);
+            r += decltype(n)::value;
+            g += 32 * decltype(n)::value;
+        };
+        while (r + kStep <= rend) step(std::integral_constant<int, kStep>());
+        if (kStep == 4 && r + 2 <= rend) step(std::integral_constant<int, 2>());
+        if (r < rend) step(std::integral_constant<int, 1>());
         ++p;
     }
 }
@@ -619,7 +625,11 @@ __device__ __forceinline__ void group_stat_flush(const ShareLaunch &a, const Sha
 // launch allocation (checked on the host against the compiled register count
 // before the shape is used: an increase the block cannot cover would wait
 // forever).
-constexpr int kWsAccRegs = 160;      // stage-2 warps: 128 accumulators
+// Stage-2 warps hold 128 accumulators: 144 registers keep enough loads in
+// flight beside them, and what they leave lets a stage-1 warp (80) issue 40
+// loads before the first use.  With 160 and 64 (32 loads) the LOFAR-like beam
+// took 6% longer; with 136 the accumulators spill (1.5 times).
+constexpr int kWsAccRegs = 144;
 constexpr int kWsStageRegs = 32;     // staging warps
 constexpr int kWsStage = 4;          // staging warps: a warpgroup
 template <int NW, int PW>
@@ -733,9 +743,10 @@ __global__ void __launch_bounds__((NW + PW + kWsStage) * 32, 1) share_ws_kernel(
                 uint32_t *P = reinterpret_cast<uint32_t *>(slot + kDmBlk);
                 share_stage1_bytes<R, CS, PW>(rec, srow, P, P + a.pmax / 2, warp, lane, xo);
             } else {
-                // 32 loads a step (no accumulators here): 8 or 4 whole rows; leftover rows in half steps
-                constexpr int kRows = 32 / CS;
-                share_stage1<Tin, R, CS, PW, kRows, kRows / 2>(rec, srow, reinterpret_cast<float *>(slot + kDmBlk), warp,
+                // 40 loads a step (no accumulators here): 10 or 5 whole rows;
+                // leftover rows 3 or 2 a step
+                constexpr int kRows = 40 / CS;
+                share_stage1<Tin, R, CS, PW, kRows, (kRows + 3) / 4>(rec, srow, reinterpret_cast<float *>(slot + kDmBlk), warp,
                                                                lane, xo);
             }
             if (warp == PW - 1)
