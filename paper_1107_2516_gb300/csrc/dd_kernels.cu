@@ -450,14 +450,16 @@ __device__ __forceinline__ void put_candidate(dd_candidate *cands, int64_t cap, 
 // Any widths: thread = kSearchPer consecutive samples.  For the widths in
 // ascending order it extends B_w at its first sample from the previous
 // width's sum, then slides it along its samples (B_w(t+1) = B_w(t) + x[t+w] -
-// x[t]); its own samples x[t] stay in registers.  17 samples a thread: an odd
+// x[t]); its own samples x[t] stay in registers.  25 samples a thread: an odd
 // stride, so that the threads' words fall in distinct banks without padding
 // and every shared address is the thread's base plus a constant or the width
 // (with 16 samples and a pad word after each 16, index arithmetic was most of
-// the kernel's instructions, and each sample and width was compared): 600
-// rows x 253 443 samples, widths 1, 3, 7, 20, 50, 0.70 -> 0.28 ms.
-constexpr int kSearchThreads = 256;
-constexpr int kSearchPer = 17;
+// the kernel's instructions, and each sample and width was compared).  600
+// rows x 253 443 samples, widths 1, 3, 7, 20, 50: 0.70 -> 0.22 ms (0.28 with
+// 17 samples and 256 threads: the first sums of the widths, 50 adds a thread,
+// are shared by fewer samples; 0.22 with 33).
+constexpr int kSearchThreads = 128;
+constexpr int kSearchPer = 25;
 constexpr int kSearchTile = kSearchThreads * kSearchPer;
 constexpr int kHitList = 1024;      // hits a block finishes per round
 static_assert(kMaxWidths <= 64, "a hit's code holds its width in 6 bits");

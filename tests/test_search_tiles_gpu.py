@@ -1,5 +1,5 @@
-"""The search kernels at the edges of their tiles and runs (4096 samples a
-block, 32 or 16 a thread), with few, many and almost all samples above the
+"""The search kernels at the edges of their tiles and runs (4096 or 3200 samples
+a block, 32 or 25 a thread), with few, many and almost all samples above the
 threshold (more than a block's hit list holds), and the finalisation over one
 and several blocks of partial statistics.  The buffers hold small whole
 numbers, so every boxcar sum is exact in float32 and the candidates are those
@@ -42,7 +42,7 @@ def run(x, widths, sigma, dtype, rows=False):
 
 
 @pytest.mark.parametrize("dtype", [dd.DD_F32, dd.DD_U8])
-@pytest.mark.parametrize("nout", [64, 65, 127, 4095, 4096, 4097, 4159, 8192 + 31])
+@pytest.mark.parametrize("nout", [64, 65, 127, 3199, 3200, 3201, 3263, 4095, 4096, 4097, 4159, 8192 + 31])
 @pytest.mark.parametrize("sigma", [3.0, -0.5])
 def test_candidates_at_tile_edges(nout, sigma, dtype):
     rng = np.random.default_rng(nout)
