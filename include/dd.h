@@ -223,9 +223,10 @@ DD_API int dd_plan_autotune(dd_plan *plan, const void *in_dev, int64_t in_pitch,
  * trials per warp, warps) — 7: 20 x 4, 8 warps; 8: 12 x 8, 8 warps; kernel
  * 5 (samples per lane x DM trials per warp, warps; 4-channel subbands) — 9:
  * 16 x 8, 4 warps; 10: 8 x 8, 4 warps; 11: 16 x 8, 6 warps; 12: 16 x 8, 8
- * warps that add the partial sums beside 8 warps that form them (one block
- * per SM, the two groups joined by mbarriers; available where the GPU's
- * compiled register count covers the split)};
+ * warps that add the partial sums beside 8 warps that form them and 4 that
+ * stage the input (one block per SM, the groups joined by mbarriers;
+ * subbands of 4 or 8 channels; input rows may start anywhere; available where
+ * the GPU's compiled register count covers the split)};
  * raster_group (>= 1) is the number of DM blocks whose time tiles are swept
  * together.  DD_ERR_ARG if the configuration cannot run this plan. */
 DD_API int dd_plan_set_tile(dd_plan *plan, int32_t config, int32_t raster_group);
@@ -290,7 +291,9 @@ DD_API int dd_batch_autotune(dd_batch *batch, const void *const *in_devs, const 
 DD_API int dd_host_chunk_schedule(int64_t nsamp_out, int64_t pitch, int32_t tile, int64_t reach,
                                   int64_t *col_end, int64_t *tile_end, int32_t *n);
 
-/* Kernel 5's tables for tile configuration `config` (9-12) of a delay table
+/* Kernel 5's tables for tile configuration `config` (9-12; 12 in the form with
+ * 4-channel subbands and float sums, what it runs with is
+ * dd_share_ws_tables') of a delay table
  * delays[ndm][nchans] (dd_plan_info's copy), computed on the host (no device
  * needed), for inspection and tests.  info[6] receives {1 if the shape can
  * run the table (at most 16 delay patterns per block and subband) else 0,

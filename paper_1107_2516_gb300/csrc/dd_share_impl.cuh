@@ -16,18 +16,19 @@
 //            its trials need (P, double-buffered in shared memory).  The
 //            patterns' sums are laid end to end in one index space e < E,
 //            cut into rows of 32 (each row inside one pattern), and each warp
-//            sums the contiguous run of rows the table assigns it, four rows
-//            per step: the pattern's fields are uniform in the warp and
+//            sums the contiguous run of rows the table assigns it, several
+//            rows per step: the pattern's fields are uniform in the warp and
 //            reloaded only where a pattern ends, and every warp gets the same
 //            number of rows;
 //   stage 2: each warp adds, for its trials, P_pat[t + offset] (one
 //            conflict-free shared word per add, as kernel 3).
-// One __syncthreads per subband: stage 1 of subband s+1 writes the other P
-// buffer while stage 2 of s reads this one; each warp takes its trials'
-// offsets into registers during stage 1 (the stage's record may be reused by
-// the next TMA copy before stage 2 ends).  The input ring has NS stages:
-// NS - 1 subbands' copies are in flight while one is summed.  The tile body
-// (share_tile) serves the one-plan kernel and the persistent batch kernel.
+// One-barrier shapes (share_tile): one __syncthreads per subband; stage 1 of
+// subband s+1 writes the other P buffer while stage 2 of s reads this one;
+// each warp takes its trials' offsets into registers during stage 1 (the
+// stage's record may be reused by the next copy before stage 2 ends).  The
+// input ring has NS stages: NS - 1 subbands' copies are in flight while one is
+// summed.  The tile body serves the one-plan kernel and the persistent batch
+// kernel.  Warp-specialised shape: share_ws_kernel below.
 #pragma once
 
 #include "dd_lane_impl.cuh"
@@ -189,7 +190,7 @@ __device__ __forceinline__ void share_stage1(const int32_t *rec, const Tin *srow
 // Stage 1 on bytes: lane l sums the four consecutive sums (a quad) of element
 // l of each of its rows of 32 quads.  Channel c's four bytes start anywhere in
 // a word: two word loads, one funnel shift, and their even and odd bytes are
-// added as pairs of 16-bit sums (at most 8 x 255).  Stage 2 reads pairs of
+// added as pairs of 16-bit sums (whole numbers of at most 8 x 255: exact).  Stage 2 reads pairs of
 // sums (u, u + 1) at any u, so P is stored twice, as pairs from even u (Pe)
 // and from odd u (Po); the pair that ends in the next quad takes that quad's
 // first sum from the bytes behind the four, one permute per two channels.
@@ -673,7 +674,7 @@ __device__ __forceinline__ bool mbar_done(uint64_t *bar, uint32_t parity)
 // the 5 copies of a subband it took 1277 of the subband's 2546 cycles on the
 // LOFAR-like plan, and everything waited for that warp's rows.  Four warps of
 // their own issue 1 to 3 copies each and are never waited for (626 of 2361
-// cycles; 888 of 2895 with 8 rows).  Measured against it: 16-byte cp.async by
+// cycles; 888 of 2895 with 8 rows; 133.1 -> 127.7 ms for the whole plan's call).  Measured against it: 16-byte cp.async by
 // the stage-2 threads (731 cycles a subband on the critical side) or by the
 // staging warps (1102; the copies then also take the loads' path into shared
 // memory: 31.9 against 30.5 ms on a quarter of the LOFAR-like plan).
