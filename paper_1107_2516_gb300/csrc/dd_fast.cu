@@ -33,6 +33,8 @@ struct LaneCfgData {
     bool ok = false;
     int ti = 0, dr = 0, nw = 0;
     int nblk = 0, rs = 0, ch = 0, bar_off = 0;
+    int ch_any = 0, bar_off_any = 0;   // the same for rows that start anywhere (ch_any 0: that form does not fit)
+    size_t smem_any = 0;
     int64_t reach = 0;           // input columns a tile at t0 reads lie below t0 + reach
     size_t smem = 0;
     int32_t *d_offs = nullptr;   // [nblk][nchans][nw*dr] offsets within the staged row
@@ -169,6 +171,10 @@ static int build_lane(const dd_plan *p, int ti, int dr, int nw, int minb, LaneCf
     if (ch < 1) return DD_OK;
     c.bar_off = (int)(((size_t)kStages * ch * per_ch + 15) / 16 * 16);
     c.smem = (size_t)c.bar_off + kStages * sizeof(uint64_t);
+    c.ch_any = (int)std::min<size_t>(16, budget / (kStages * (per_ch + 16)));   // rows one 16-byte unit longer
+    if (fours) c.ch_any = c.ch_any / 4 * 4;
+    c.bar_off_any = (int)(((size_t)kStages * c.ch_any * (per_ch + 16) + 15) / 16 * 16);
+    c.smem_any = (size_t)c.bar_off_any + kStages * sizeof(uint64_t);
     c.reach = (int64_t)*std::max_element(base.begin(), base.end()) + rs;
     c.nblk = nblk; c.rs = rs; c.ch = ch;
     cudaError_t e = cudaMalloc(&c.d_offs, offs.size() * 4);
@@ -753,6 +759,7 @@ int fast_configure(dd_plan *p)
     for (int k = 0; k < kNumLaneCfg && rc == DD_OK && e == cudaSuccess; ++k)
         if (f->lane[k].ok) e = prepare_lane(k, p->smem_optin);
     if (rc == DD_OK && e == cudaSuccess && f->small.ok) e = lane_prepare_small(p->smem_optin);
+    if (rc == DD_OK && e == cudaSuccess && (f->small.ok || f->lane[kLaneAny].ok)) e = lane_prepare_any(p->smem_optin);
     for (int k = 0; k < kNumTmemCfg && rc == DD_OK && e == cudaSuccess; ++k)
         if (f->tm[k].ok) e = prepare_tmem(k, p->smem_optin);
     for (int k = 0; k < kNumShareCfg && rc == DD_OK && e == cudaSuccess; ++k)
@@ -786,6 +793,12 @@ int fast_error(dd_plan *p, cudaStream_t s)
     return DD_OK;
 }
 
+// Whether input rows start on 16-byte boundaries, as the tiled kernels' bulk copies need.
+static bool rows_aligned(const FastPlan *f, const void *in, int64_t pitch)
+{
+    return !((uintptr_t)in & 15u) && pitch % f->al == 0;
+}
+
 // Partial-statistics record size of the plan's input type.
 static size_t stat_bytes(const dd_plan *p) { return p->dtype == DD_U8 ? sizeof(StatI) : sizeof(StatF); }
 
@@ -815,7 +828,15 @@ static int lane_run(dd_plan *p, int k, int dgroup, const void *in, int64_t pitch
     a.dgroup = std::max(1, std::min(dgroup, c.nblk));
     a.out = out; a.err = f->d_err; a.smem = c.smem;
     a.partials = static_cast<char *>(p->d_partials) + (size_t)(tile_lo * c.nblk) * stat_bytes(p);
-    cudaError_t e = small ? lane_launch_small(p->dtype, a, f->active >= kShareBeg, s) : launch_lane(k, p->dtype, a, s);
+    const bool any = !rows_aligned(f, in, pitch);
+    if (any) {      // k is kLaneAny or kLaneSmall: fast_execute
+        a.in_res = (int)((uintptr_t)in / in_elem_bytes(p->dtype) % f->al);
+        a.nsamp_in_al = p->nsamp_in;
+        a.rs = c.rs + f->al; a.ch = c.ch_any; a.bar_off = c.bar_off_any; a.smem = c.smem_any;
+    }
+    const bool fours = f->active >= kShareBeg;
+    cudaError_t e = any ? lane_launch_any(p->dtype, a, small, fours, s)
+                  : small ? lane_launch_small(p->dtype, a, fours, s) : launch_lane(k, p->dtype, a, s);
     if (e != cudaSuccess) return cuda_fail(e, "launch lane_kernel");
     p->n_partials = np;
     p->stats_out = out;
@@ -845,12 +866,6 @@ static int tmem_run(dd_plan *p, int k, int dgroup, const void *in, int64_t pitch
     p->n_partials = np;
     p->stats_out = out;
     return DD_OK;
-}
-
-// Whether input rows start on 16-byte boundaries, as the tiled kernels' bulk copies need.
-static bool rows_aligned(const FastPlan *f, const void *in, int64_t pitch)
-{
-    return !((uintptr_t)in & 15u) && pitch % f->al == 0;
 }
 
 // Kernel 5 on output tiles [tile_lo, tile_hi), as lane_run.
@@ -926,15 +941,23 @@ int fast_execute(dd_plan *p, const void *in, int64_t pitch, void *out, cudaStrea
     FastPlan *f = static_cast<FastPlan *>(p->fast);
     if (!f) return set_error(DD_ERR_ARG, "kernel 2 unavailable for this plan");
     // Bulk copies need 16-byte aligned rows; for other rows the warp-specialised
-    // kernel 5 stages whole units around them (a cut of 200 channels x 150001
-    // samples, 301 trials: 3.77 ms on the generic kernel, 0.61 ms here), and
-    // where its tables do not fit the generic kernel runs.
+    // kernel 5 and kernel 3 (plans whose tables kernel 5 does not take) stage
+    // whole units around them, and where neither fits the generic kernel runs:
+    // 200 channels x 150001 samples, 301 trials: 3.77 ms on the generic kernel,
+    // 0.61 ms on kernel 5; 64 channels, 41 trials x 150001 samples: 166 us on
+    // the generic kernel, 86 us on kernel 3 (float16 138 and 87, uint8 123 and
+    // 83), x 8191 samples in its finer shape 54 and 13 us (uint8 48 and 11); 1024
+    // channels, 64 trials x 8191 samples: 256 us on kernel 5, 103 us in the finer
+    // shape (uint8 182 and 95).
     if (!rows_aligned(f, in, pitch)) {
-        const int k = kShareBeg + kShareWs;
-        if (f->active < kShareBeg || !f->sh[kShareWs].ok || !f->sh[kShareWs].ns_any ||
-            (uintptr_t)in % in_elem_bytes(p->dtype))
-            return generic_execute(p, in, pitch, out, s);
-        return fast_run(p, k, f->dgroup, in, pitch, out, s);
+        const bool whole = (uintptr_t)in % in_elem_bytes(p->dtype) == 0;
+        if (whole && f->small.ok && f->small.ch_any && !f->forced && few_blocks(p, f))
+            return lane_run(p, -1, f->dgroup, in, pitch, out, s);
+        if (whole && f->active >= kShareBeg && f->sh[kShareWs].ok && f->sh[kShareWs].ns_any)
+            return fast_run(p, kShareBeg + kShareWs, f->dgroup, in, pitch, out, s);
+        if (whole && f->active >= kNumFastCfg && f->active < kLaneEnd && f->lane[kLaneAny].ok && f->lane[kLaneAny].ch_any)
+            return lane_run(p, kLaneAny, f->dgroup, in, pitch, out, s);
+        return generic_execute(p, in, pitch, out, s);
     }
     if (f->small.ok && !f->forced && few_blocks(p, f)) return lane_run(p, -1, f->dgroup, in, pitch, out, s);
     return fast_run(p, f->active, f->dgroup, in, pitch, out, s);

@@ -34,6 +34,7 @@ struct LaneLaunch {
     int dtype;             // dd_dtype of `in` (batched launches)
     int64_t t_base;        // lane_kernel: first output sample of the launch's tile range
     int kind;              // mixed batch: 0 = this kernel 3 launch, 1 = the beam's kernel 5 launch
+    int in_res;            // rows that start anywhere: element of its 16-byte unit that `in` points at
 };
 
 template <typename Tin> __device__ __forceinline__ float lane_ld(const Tin *p);
@@ -66,9 +67,9 @@ struct ByteSums {
     }
 
     // M channels: their staged rows from `rows` on, rs apart; this warp's
-    // trials' offsets from `so` on, os apart.
-    template <int M>
-    __device__ __forceinline__ void add(const uint8_t *rows, int rs, const int32_t *so, int os, int lane)
+    // trials' offsets from `so` on, os apart, plus xo(c).
+    template <int M, typename X>
+    __device__ __forceinline__ void add(const uint8_t *rows, int rs, const int32_t *so, int os, int lane, X xo)
     {
         constexpr uint32_t kEven = 0x00ff00ffu;
         const uint32_t *w = reinterpret_cast<const uint32_t *>(rows) + lane;
@@ -79,7 +80,8 @@ struct ByteSums {
 #pragma unroll
             for (int c = 0; c < M; ++c) {
                 const int4 v = *reinterpret_cast<const int4 *>(so + c * os + q);
-                o[c][0] = v.x; o[c][1] = v.y; o[c][2] = v.z; o[c][3] = v.w;
+                const int x = xo(c);
+                o[c][0] = v.x + x; o[c][1] = v.y + x; o[c][2] = v.z + x; o[c][3] = v.w + x;
             }
 #pragma unroll
             for (int j = 0; j < 4; ++j)
@@ -101,11 +103,12 @@ struct ByteSums {
         }
     }
 
-    __device__ __forceinline__ void add_stage(const uint8_t *rows, int rs, const int32_t *so, int os, int cn, int lane)
+    template <typename X>
+    __device__ __forceinline__ void add_stage(const uint8_t *rows, int rs, const int32_t *so, int os, int cn, int lane, X xo)
     {
         int c = 0;
-        for (; c + 4 <= cn; c += 4) add<4>(rows + (size_t)c * rs, rs, so + c * os, os, lane);
-        for (; c < cn; ++c) add<1>(rows + (size_t)c * rs, rs, so + c * os, os, lane);
+        for (; c + 4 <= cn; c += 4) add<4>(rows + (size_t)c * rs, rs, so + c * os, os, lane, [&](int k) { return xo(c + k); });
+        for (; c < cn; ++c) add<1>(rows + (size_t)c * rs, rs, so + c * os, os, lane, [&](int k) { return xo(c + k); });
     }
 
     // sum of sample 4 l + 128 i + e
@@ -139,8 +142,9 @@ __device__ __forceinline__ void lane_raster(const LaneLaunch &a, int64_t lin, in
 // call.
 // kFours (ch a multiple of 4, nchans too): four channels are summed before
 // they are added, kernel 5's order with subbands of 4 and so its float sums to
-// the bit.
-template <typename Tin, bool kInt, int TI, int DR, int NW, bool kFours = false>
+// the bit.  kAny: rows that start anywhere, staged as in share_ws_kernel: whole
+// 16-byte units around a row's samples, in rows one unit longer.
+template <typename Tin, bool kInt, int TI, int DR, int NW, bool kFours = false, bool kAny = false>
 __device__ __forceinline__ bool lane_tile(const LaneLaunch &a, int blk, int64_t t0, int64_t lin,
                                           uint64_t *bar, uint32_t &gstage)
 {
@@ -167,15 +171,24 @@ __device__ __forceinline__ bool lane_tile(const LaneLaunch &a, int blk, int64_t 
     // the subband kernel, which has the same body, took 12.06 and 10.03 ms for
     // its stages of the LOFAR-like plan and takes 10.87 and 8.17).  The row's
     // start is loaded one stage early.
+    constexpr int kAl = 16 / (int)sizeof(Tin);
+    const int pitch_res = (int)(a.pitch & (kAl - 1));
+    auto res = [&](int c) { return kAny ? (a.in_res + c * pitch_res) & (kAl - 1) : 0; };
     const int mine = warp + NW * lane;
     int rb = mine < ch ? bbase[min(mine, nchans - 1)] : 0;   // of the next stage to issue
     auto issue = [&](int s) {
         const int buf = (int)((g0 + s) % kStages);
         const int c0 = s * ch;
         const int cn = min(ch, nchans - c0);
-        const int64_t g = t0 + rb;
+        const int most = kAny ? rs - kAl : rs;
+        int64_t g = t0 + rb;
         int64_t n = a.nsamp_in_al - g;
-        n = n < 0 || mine >= cn ? 0 : (n > rs ? rs : n);
+        n = n < 0 || mine >= cn ? 0 : (n > most ? most : n);
+        if (kAny && n > 0) {
+            const int d = res(c0 + mine);
+            n = (n + d + kAl - 1) & ~(int64_t)(kAl - 1);
+            g -= d;
+        }
         const uint32_t nb = (uint32_t)(n * (int64_t)sizeof(Tin)), ob = (uint32_t)(cn * kDmBlk * sizeof(int32_t));
         const uint32_t bytes = __reduce_add_sync(0xffffffffu, nb) + (warp == NW - 1 ? ob : 0u);
         if (lane == 0) {
@@ -214,7 +227,8 @@ __device__ __forceinline__ bool lane_tile(const LaneLaunch &a, int blk, int64_t 
         const int cn = idle ? 0 : min(ch, nchans - s * ch);
         const Tin *srow = rows + (size_t)buf * stage_elems + lane;
         const int32_t *so = soffs + (size_t)buf * ch * kDmBlk + warp * DR;
-        if constexpr (kBytes) bs.add_stage(srow - lane, rs, so, kDmBlk, cn, lane);
+        const int c0 = s * ch;
+        if constexpr (kBytes) bs.add_stage(srow - lane, rs, so, kDmBlk, cn, lane, [&](int c) { return res(c0 + c); });
         else if constexpr (kFours) for (int cc = 0; cc < cn; cc += 4) {
             const Tin *r = srow + (size_t)cc * rs;
 #pragma unroll
@@ -223,7 +237,8 @@ __device__ __forceinline__ bool lane_tile(const LaneLaunch &a, int blk, int64_t 
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     const int4 v = *reinterpret_cast<const int4 *>(so + (cc + c) * kDmBlk + j);
-                    o[0][c] = v.x; o[1][c] = v.y; o[2][c] = v.z; o[3][c] = v.w;
+                    const int x = res(c0 + cc + c);
+                    o[0][c] = v.x + x; o[1][c] = v.y + x; o[2][c] = v.z + x; o[3][c] = v.w + x;
                 }
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
@@ -237,7 +252,7 @@ __device__ __forceinline__ bool lane_tile(const LaneLaunch &a, int blk, int64_t 
             }
         }
         else for (int cc = 0; cc < cn; ++cc) {
-            const Tin *r = srow + (size_t)cc * rs;
+            const Tin *r = srow + (size_t)cc * rs + res(c0 + cc);
             // the warp's DR offsets: uniform 16-byte loads, one shared-memory
             // wavefront per 4 offsets (the data path is the kernel's bound)
             int o[DR];
@@ -313,7 +328,7 @@ __device__ __forceinline__ bool lane_tile(const LaneLaunch &a, int blk, int64_t 
 }
 
 // One plan: one block per work item, grid = nblk * ntile.
-template <typename Tin, bool kInt, int TI, int DR, int NW, int MINB, bool kFours = false>
+template <typename Tin, bool kInt, int TI, int DR, int NW, int MINB, bool kFours = false, bool kAny = false>
 __global__ void __launch_bounds__(NW * 32, MINB) lane_kernel(LaneLaunch a)
 {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -328,7 +343,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) lane_kernel(LaneLaunch a)
     lane_raster<TI>(a, blockIdx.x, blk, t0);
     t0 += a.t_base;
     uint32_t gstage = 0;
-    lane_tile<Tin, kInt, TI, DR, NW, kFours>(a, blk, t0, blockIdx.x, bar, gstage);
+    lane_tile<Tin, kInt, TI, DR, NW, kFours, kAny>(a, blk, t0, blockIdx.x, bar, gstage);
 }
 
 // lane_tile as an out-of-line function: the persistent kernel calls one per
@@ -389,26 +404,26 @@ __global__ void __launch_bounds__(NW * 32, MINB) lane_batch_kernel(LaneBatchLaun
     }
 }
 
-template <int TI, int DR, int NW, int MINB, bool kFours = false>
+template <int TI, int DR, int NW, int MINB, bool kFours = false, bool kAny = false>
 cudaError_t lane_launch_cfg(dd_dtype t, const LaneLaunch &a, cudaStream_t s)
 {
     const unsigned grid = (unsigned)(a.ntile * a.nblk);
     switch (t) {
-    case DD_F32: lane_kernel<float, false, TI, DR, NW, MINB, kFours><<<grid, NW * 32, a.smem, s>>>(a); break;
-    case DD_F16: lane_kernel<__half, false, TI, DR, NW, MINB, kFours><<<grid, NW * 32, a.smem, s>>>(a); break;
-    case DD_U8: lane_kernel<uint8_t, true, TI, DR, NW, MINB><<<grid, NW * 32, a.smem, s>>>(a); break;
+    case DD_F32: lane_kernel<float, false, TI, DR, NW, MINB, kFours, kAny><<<grid, NW * 32, a.smem, s>>>(a); break;
+    case DD_F16: lane_kernel<__half, false, TI, DR, NW, MINB, kFours, kAny><<<grid, NW * 32, a.smem, s>>>(a); break;
+    case DD_U8: lane_kernel<uint8_t, true, TI, DR, NW, MINB, false, kAny><<<grid, NW * 32, a.smem, s>>>(a); break;
     }
     return cudaGetLastError();
 }
 
-template <int TI, int DR, int NW, int MINB, bool kFours = false>
+template <int TI, int DR, int NW, int MINB, bool kFours = false, bool kAny = false>
 cudaError_t lane_prepare_one(size_t optin)
 {
-    cudaError_t e = allow_max_dynamic_smem((const void *)lane_kernel<float, false, TI, DR, NW, MINB, kFours>, optin);
+    cudaError_t e = allow_max_dynamic_smem((const void *)lane_kernel<float, false, TI, DR, NW, MINB, kFours, kAny>, optin);
     if (e == cudaSuccess)
-        e = allow_max_dynamic_smem((const void *)lane_kernel<__half, false, TI, DR, NW, MINB, kFours>, optin);
+        e = allow_max_dynamic_smem((const void *)lane_kernel<__half, false, TI, DR, NW, MINB, kFours, kAny>, optin);
     if (e == cudaSuccess)
-        e = allow_max_dynamic_smem((const void *)lane_kernel<uint8_t, true, TI, DR, NW, MINB>, optin);
+        e = allow_max_dynamic_smem((const void *)lane_kernel<uint8_t, true, TI, DR, NW, MINB, false, kAny>, optin);
     return e;
 }
 
@@ -442,6 +457,10 @@ constexpr LaneShape kLaneCfg[kNumLaneCfg] = {{16, 4, 8, 2}, {16, 8, 8, 1}, {16, 
 constexpr LaneShape kLaneSmall = {4, 4, 4, 4};
 cudaError_t lane_launch_small(dd_dtype t, const LaneLaunch &a, bool fours, cudaStream_t s);
 cudaError_t lane_prepare_small(size_t optin);
+// Rows that start anywhere: shape kLaneAny or (small; fours: kFours) kLaneSmall.
+constexpr int kLaneAny = 2;
+cudaError_t lane_launch_any(dd_dtype t, const LaneLaunch &a, bool small, bool fours, cudaStream_t s);
+cudaError_t lane_prepare_any(size_t optin);
 
 cudaError_t lane_launch_c0(dd_dtype t, const LaneLaunch &a, cudaStream_t s);
 cudaError_t lane_launch_c1(dd_dtype t, const LaneLaunch &a, cudaStream_t s);

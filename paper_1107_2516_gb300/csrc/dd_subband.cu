@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(NW * 32, 3) sub_kernel(SubLaunch a)
         const int cn = idle ? 0 : min(ch, nchans - s * ch);
         const Tin *srow = rows + (size_t)buf * stage_elems + lane;
         const int32_t *so = soffs + (size_t)buf * ch * kDmBlk + warp * DR;
-        if constexpr (kBytes) bs.add_stage(srow - lane, rs, so, kDmBlk, cn, lane);
+        if constexpr (kBytes) bs.add_stage(srow - lane, rs, so, kDmBlk, cn, lane, [](int) { return 0; });
         else for (int cc = 0; cc < cn; ++cc) {
             const Tin *r = srow + (size_t)cc * rs;
             int o[DR];

@@ -91,3 +91,37 @@ def test_launches_of_few_blocks_give_the_same_sums(case, dtype):
         plan.close()
     assert np.array_equal(got[0][0], got[1][0]) and np.all(got[0][0][-16:] == -7)
     assert got[0][1] == pytest.approx(got[1][1], rel=1e-5, abs=1e-5)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "u8", "f16"])
+@pytest.mark.parametrize("nch,step,kernel", [(65, 0.1, 3), (64, 0.01, 5)])
+@pytest.mark.parametrize("off,pad", [(0, 1), (3, 5), (1, 7), (2, None)])
+def test_rows_that_start_anywhere_on_kernel_3(off, pad, nch, step, kernel, dtype):
+    # a plan by itself (few blocks: the finer shape, in kernel 5's order if that is its kernel) and
+    # with a shape of kernel 3 chosen
+    fch1, foff, ts, dms = 150.0, -0.39, 327.68e-6, [step * i for i in range(41)]
+    d, m = oracle.delays(nch, fch1, foff, ts, dms)
+    al = 16 // {"f32": 4, "u8": 1, "f16": 2}[dtype]
+    for nout in (1, 127, 513, 1100):
+        nsamp = nout + m
+        pitch = nsamp + pad if pad is not None else -(-nsamp // al) * al
+        x = synth.noise_f32(nch, nsamp, 5)
+        x = synth.quantize_u8(x) if dtype == "u8" else x.astype(np.float16) if dtype == "f16" else x
+        flat = np.full(off + (nch - 1) * pitch + nsamp, 99, x.dtype)     # the last row ends with its samples
+        for c in range(nch):
+            flat[off + c * pitch:off + c * pitch + nsamp] = x[c]
+        dev = torch.from_numpy(flat.view(np.int16) if dtype == "f16" else flat).cuda()
+        ref = oracle.dedisperse(x if dtype == "u8" else x.astype(np.float32), np.asarray(d), nout)
+        for forced in (False, True):
+            plan = dd.Plan(nch, fch1, foff, ts, dms, [1], 6.0, TYPE[dtype], nsamp)
+            assert plan.kernel == kernel
+            if forced:
+                plan.set_tile(5, 8)
+            out = torch.full((len(dms) * nout + 32,), -7, dtype=torch.int32 if dtype == "u8" else torch.float32, device="cuda")
+            plan.execute(dev.data_ptr() + off * flat.itemsize, pitch, out)
+            plan.search(out, allow_overflow=True)
+            got = out.cpu().numpy()
+            plan.close()
+            assert np.all(got[-32:] == -7)
+            got = got[:-32].reshape(len(dms), nout)
+            assert np.array_equal(got, ref) if dtype == "u8" else np.max(np.abs(got - ref)) <= 1e-5 * nch
