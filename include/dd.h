@@ -264,7 +264,8 @@ DD_API int dd_batch_execute(dd_batch *batch, const void *const *in_devs, const i
 
 /* Record dd_batch_execute's work for these buffers as a CUDA graph (stream
  * capture on `stream`); dd_batch_launch then replays it.  Allocates what the
- * launches need before capturing. */
+ * launches need before capturing; the graph stays valid while the plans are
+ * also used alone. */
 DD_API int dd_batch_capture(dd_batch *batch, const void *const *in_devs, const int64_t *in_pitches,
                             void *const *out_devs, void *stream);
 

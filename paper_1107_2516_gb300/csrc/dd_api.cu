@@ -69,6 +69,7 @@ static void free_plan(dd_plan *p)
     fast_release(p);
     if (p->d_gen) cudaFree(p->d_gen);
     if (p->d_partials) cudaFree(p->d_partials);
+    for (void *q : p->old_partials) cudaFree(q);
     if (p->d_back) cudaFree(p->d_back);
     if (p->d_fin) cudaFree(p->d_fin);
     if (p->d_wsorted) cudaFree(p->d_wsorted);

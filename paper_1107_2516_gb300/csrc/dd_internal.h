@@ -91,6 +91,7 @@ struct dd_plan {
     // statistics partials of the last dd_execute
     void *d_partials = nullptr;            // StatF or StatI per block
     int64_t n_partials_cap = 0;
+    std::vector<void *> old_partials;      // outgrown buffers: captured graphs may still use them
     int64_t n_partials = 0;
     const void *stats_out = nullptr;       // out buffer the partials describe
     // search

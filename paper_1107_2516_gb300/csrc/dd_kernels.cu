@@ -872,12 +872,17 @@ cudaError_t allow_max_dynamic_smem(const void *fn, size_t optin)
 int ensure_partials_public(dd_plan *p, int64_t n)
 {
     if (n <= p->n_partials_cap) return DD_OK;
-    if (p->d_partials) cudaFree(p->d_partials);
-    p->d_partials = nullptr;
-    p->n_partials_cap = 0;
-    cudaError_t e = cudaMalloc(&p->d_partials, (size_t)n * stat_size(p));
+    // An outgrown buffer stays until the plan goes: a graph captured before (a
+    // batch's, or a caller's own) holds its address, and its kernels write and
+    // read their partials there.  Shapes differ in their number of blocks (the
+    // finer shape of a launch of few blocks has 8 times the others'), so a plan
+    // outgrows its buffer at most once per shape.
+    void *q = nullptr;
+    cudaError_t e = cudaMalloc(&q, (size_t)n * stat_size(p));
     if (e != cudaSuccess) return set_error(DD_ERR_NOMEM, "cudaMalloc(partials, %lld): %s",
                                            (long long)n, cudaGetErrorString(e));
+    if (p->d_partials) p->old_partials.push_back(p->d_partials);
+    p->d_partials = q;
     p->n_partials_cap = n;
     return DD_OK;
 }
