@@ -447,27 +447,51 @@ __device__ __forceinline__ void put_candidate(dd_candidate *cands, int64_t cap, 
     cands[pos] = c;
 }
 
-// Any widths: thread = kSearchPer consecutive samples.  For the widths in
-// ascending order it extends B_w at its first sample from the previous
-// width's sum, then slides it along its samples (B_w(t+1) = B_w(t) + x[t+w] -
-// x[t]); its own samples x[t] stay in registers.  25 samples a thread: an odd
+// Any widths: thread = kPer consecutive samples.  For the widths in ascending
+// order it extends B_w at its first sample from the previous width's sum, then
+// slides it along its samples (B_w(t+1) = B_w(t) + x[t+w] - x[t]); its own
+// samples x[t] stay in registers.  31 samples a thread (25 integers): an odd
 // stride, so that the threads' words fall in distinct banks without padding
 // and every shared address is the thread's base plus a constant or the width
 // (with 16 samples and a pad word after each 16, index arithmetic was most of
-// the kernel's instructions, and each sample and width was compared).  600
-// rows x 253 443 samples, widths 1, 3, 7, 20, 50: 0.70 -> 0.22 ms (0.28 with
-// 17 samples and 256 threads: the first sums of the widths, 50 adds a thread,
-// are shared by fewer samples; 0.22 with 33).
+// the kernel's instructions, and each sample and width was compared).
+//
+// Every slide of a floating-point sum rounds, and a sample that swamps the sum
+// (or an infinity) spoils the windows behind it until the next sum formed
+// afresh.  So a run of 31 has two: 15 slides at most, as in runs of 16.  (One
+// per 25 samples: r.m.s. error on noise 1.05 to 1.24 times that of runs of 16;
+// now 0.98 of it.)  Integers slide through the whole run.
+//
+// A width more than kSearchGap above the previous one starts from the sums of
+// the half runs it covers (16 and 15 samples, formed once) with at most 15
+// single samples behind them: 3000 samples take 208 adds, and round less than
+// one by one.
+//
+// 600 rows x 253 443 float32 samples without hits: widths 1, 3, 7, 20, 50 0.67 ms
+// with runs of 16, 0.21 with one fresh sum per 25 samples, 0.22 now; 1, 30, 300,
+// 3000 4.70, 2.03, 0.97 ms; 1 to 64 6.85, 1.39, 1.37 ms.
 constexpr int kSearchThreads = 128;
-constexpr int kSearchPer = 25;
-constexpr int kSearchTile = kSearchThreads * kSearchPer;
+constexpr int kSearchGap = 64;
+template <bool kInt>
+struct SearchShape {
+    static constexpr int kRun = kInt ? 13 : 16;        // samples of a first half run
+    static constexpr int kPer = 2 * kRun - 1;          // samples per thread
+    static constexpr int kTile = kSearchThreads * kPer;
+    // half runs of the staged samples (a tile and wmax - 1 more)
+    static __host__ __device__ constexpr int halves(int wmax) { return 2 * ((kTile + wmax - 1 + kPer - 1) / kPer); }
+    // staged samples and, for wide gaps, the half runs' sums
+    static constexpr size_t smem(int wmax, bool wide) { return (size_t)(kTile + wmax - 1 + (wide ? halves(wmax) : 0)) * 4; }
+};
+// with the kernel's own 10 or 14.4 KB within what any launch may have
+static_assert(SearchShape<false>::smem(4096, true) + 10 * 1024 <= 48 * 1024 &&
+              SearchShape<true>::smem(4096, true) + 15 * 1024 <= 48 * 1024, "no attribute to set on each call");
 constexpr int kHitList = 1024;      // hits a block finishes per round
 static_assert(kMaxWidths <= 64, "a hit's code holds its width in 6 bits");
 
 template <bool kInt>
-__global__ void __launch_bounds__(kSearchThreads)
+__global__ void __launch_bounds__(kSearchThreads, kInt ? 5 : 6)
 search_kernel(const void *__restrict__ out_, int64_t nout,
-              const int32_t *__restrict__ wsorted, int nw, int wmax,
+              const int32_t *__restrict__ wsorted, int nw, int wmax, int wide,
               const SearchParams *__restrict__ prm, const RowParams *__restrict__ rp,
               dd_candidate *__restrict__ cands, int64_t cap, unsigned long long *__restrict__ count)
 {
@@ -480,6 +504,8 @@ search_kernel(const void *__restrict__ out_, int64_t nout,
     __shared__ int hcode[kHitList];                 // sample << 6 | sorted width
     __shared__ int nlist;
     __shared__ unsigned long long first;
+    using S = SearchShape<kInt>;
+    constexpr int kSearchPer = S::kPer, kSearchRun = S::kRun, kSearchTile = S::kTile;
     T *x = reinterpret_cast<T *>(sraw);
     const int row = blockIdx.y;
     const int64_t t0 = (int64_t)blockIdx.x * kSearchTile;
@@ -516,19 +542,54 @@ search_kernel(const void *__restrict__ out_, int64_t nout,
     T own[kSearchPer];
 #pragma unroll
     for (int i = 0; i < kSearchPer; ++i) own[i] = xb[i];
-    Acc b0 = 0;          // running B_w at the thread's first sample
+    T *half = x + len;   // the sums of the half runs: 2 u at sample kPer u, 2 u + 1 kRun samples behind it
+    if (wide) {
+        T a = own[0], b = own[kSearchRun];
+#pragma unroll
+        for (int i = 1; i < kSearchRun; ++i) a += own[i];
+#pragma unroll
+        for (int i = kSearchRun + 1; i < kSearchPer; ++i) b += own[i];
+        half[2 * threadIdx.x] = a;
+        half[2 * threadIdx.x + 1] = b;
+        for (int h = 2 * kSearchThreads + threadIdx.x; h < S::halves(wmax); h += kSearchThreads) {
+            const int s = (h >> 1) * kSearchPer + (h & 1) * kSearchRun;
+            const int e = min(s + kSearchRun - (h & 1), len);
+            T v = 0;
+            for (int j = s; j < e; ++j) v += x[j];
+            half[h] = v;
+        }
+        __syncthreads();
+    }
+    // B_w at sample c * kRun of the thread's run from its whole half runs
+    auto cover = [&](int c, int w) {
+        Acc v = 0;
+        int h = 2 * threadIdx.x + c, n = 0;
+        for (int l; n + (l = kSearchRun - (h & 1)) <= w; n += l, ++h) v += (Acc)half[h];
+        for (; n < w; ++n) v += (Acc)xb[c * kSearchRun + n];
+        return v;
+    };
+    Acc b0 = 0, b1 = 0;  // B_w at the thread's first sample and (floating point) at sample kRun
     int wprev = 0;
     for (int p = 0; p < nw; ++p) {
         const int w = sw[p];
+        if (w - wprev > kSearchGap) {
+            b0 = cover(0, w);
+            if constexpr (!kInt) b1 = cover(1, w);
+        } else {
 #pragma unroll 4
-        for (int j = wprev; j < w; ++j) b0 += (Acc)xb[j];
+            for (int j = wprev; j < w; ++j) {
+                b0 += (Acc)xb[j];
+                if constexpr (!kInt) b1 += (Acc)xb[kSearchRun + j];
+            }
+        }
         wprev = w;
         const Acc thr = sthr[p];
         const T *xw = xb + (w - 1);              // xw[i] = x[base + i - 1 + w], the sample that enters at i
         Acc b = b0, m = b0;
 #pragma unroll
         for (int i = 1; i < kSearchPer; ++i) {
-            b += (Acc)xw[i] - (Acc)own[i - 1];
+            if (!kInt && i == kSearchRun) b = b1;
+            else b += (Acc)xw[i] - (Acc)own[i - 1];
             if constexpr (kInt) m = b > m ? b : m;
             else m = fmaxf(m, b);
         }
@@ -539,7 +600,8 @@ search_kernel(const void *__restrict__ out_, int64_t nout,
         for (int i = 0; i < kSearchPer; ++i) {
             const int64_t t = t0 + base + i;
             if (t + w > nout) break;
-            if (i > 0) b += (Acc)xw[i] - (Acc)xb[i - 1];
+            if (!kInt && i == kSearchRun) b = b1;
+            else if (i > 0) b += (Acc)xw[i] - (Acc)xb[i - 1];
             if (!(b > thr)) continue;
             // the list, or (full) the slow way
             const int at = atomicAdd(&nlist, 1);
@@ -1029,19 +1091,24 @@ int search_launch(dd_plan *p, const void *out, cudaStream_t s)
     int wmax = 0;
     for (int w : p->widths) wmax = std::max(wmax, w);
     const int K = pow2_widths(p);
-    const int tile = K ? kPow2Tile : kSearchTile;
+    const int tile = K ? kPow2Tile : isint ? SearchShape<true>::kTile : SearchShape<false>::kTile;
     const dim3 grid((unsigned)((p->nsamp_out + tile - 1) / tile), (unsigned)p->ndm);
-    const size_t smem = (size_t)(kSearchTile + wmax - 1) * 4;
+    int ws[kMaxWidths];
+    std::copy(p->widths.begin(), p->widths.end(), ws);
+    std::sort(ws, ws + p->nwidths);
+    bool wide = false;
+    for (int i = 0; i < p->nwidths; ++i) wide |= ws[i] - (i ? ws[i - 1] : 0) > kSearchGap;
+    const size_t smem = isint ? SearchShape<true>::smem(wmax, wide) : SearchShape<false>::smem(wmax, wide);
     if (K) {
         if (isint) launch_search_pow2_k<true>(K, grid, s, out, p);
         else launch_search_pow2_k<false>(K, grid, s, out, p);
     } else if (isint)
         search_kernel<true><<<grid, kSearchThreads, smem, s>>>(out, p->nsamp_out, p->d_wsorted, p->nwidths,
-                                                               wmax, p->d_params, rp, p->d_cands, p->cand_cap,
+                                                               wmax, wide, p->d_params, rp, p->d_cands, p->cand_cap,
                                                                p->d_count);
     else
         search_kernel<false><<<grid, kSearchThreads, smem, s>>>(out, p->nsamp_out, p->d_wsorted, p->nwidths,
-                                                                wmax, p->d_params, rp, p->d_cands, p->cand_cap,
+                                                                wmax, wide, p->d_params, rp, p->d_cands, p->cand_cap,
                                                                 p->d_count);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "launch search_kernel");
