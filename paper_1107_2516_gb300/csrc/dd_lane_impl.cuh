@@ -42,6 +42,27 @@ template <> __device__ __forceinline__ float lane_ld<float>(const float *p) { re
 template <> __device__ __forceinline__ float lane_ld<__half>(const __half *p) { return __half2float(*p); }
 template <> __device__ __forceinline__ float lane_ld<uint8_t>(const uint8_t *p) { return (float)*p; }
 
+// Swaps a bit of v's index with a bit of the lane's number.  Lanes that hold
+// four consecutive samples each (4 l + e) would store words 4 apart, and every
+// store of the warp would touch the sectors of four; afterwards each covers 32
+// consecutive samples, wherever the row starts (4 channels uint8, 200 trials x
+// 30 000 samples: 12.4 us with one sample a lane, 16.5 us with the words apart,
+// 12.4 us now).
+template <int kReg, int kLane, int N>
+__device__ __forceinline__ void swap_with_lane_bit(uint32_t (&v)[N], int lane)
+{
+    const bool up = lane & kLane;
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+        if (!(k & kReg)) {
+            const uint32_t got = __shfl_xor_sync(0xffffffffu, up ? v[k] : v[k | kReg], kLane);
+            if (up) v[k] = got;
+            else v[k | kReg] = got;
+        }
+}
+// Sample (of 32) in a lane's registers after bits 0 and 1 were swapped with the lane's bits 3 and 4.
+__device__ __forceinline__ int quad_sample(int lane) { return 4 * (lane & 7) + (lane >> 3); }
+
 // Sums of bytes, four consecutive samples a step: lane l owns samples 4 l + 128
 // i + e (i < TI / 4, e < 4).  A trial's four bytes start anywhere in a word:
 // two word loads and a funnel shift, then their even and odd bytes are added
@@ -111,10 +132,13 @@ struct ByteSums {
         for (; c < cn; ++c) add<1>(rows + (size_t)c * rs, rs, so + c * os, os, lane, [&](int k) { return xo(c + k); });
     }
 
-    // sum of sample 4 l + 128 i + e
-    __device__ __forceinline__ uint32_t at(int j, int i, int e) const
+    // The sums of trial j's samples 128 i on: v[k] that of sample 128 i + 32 k + quad_sample(lane).
+    __device__ __forceinline__ void at(int j, int i, int lane, uint32_t (&v)[4]) const
     {
-        return e >= 2 ? h[j][i][e & 1] : a[j][i][e] - (h[j][i][e] << 16);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = e >= 2 ? h[j][i][e & 1] : a[j][i][e] - (h[j][i][e] << 16);
+        swap_with_lane_bit<1, 8>(v, lane);
+        swap_with_lane_bit<2, 16>(v, lane);
     }
 };
 
@@ -281,17 +305,21 @@ __device__ __forceinline__ bool lane_tile(const LaneLaunch &a, int blk, int64_t 
         long long n = 0, s = 0;
         unsigned long long q = 0;
         int32_t *out = reinterpret_cast<int32_t *>(a.out);
+        const int left = (int)min(nout - t0 - quad_sample(lane), (int64_t)32 * TI);
 #pragma unroll
         for (int j = 0; j < DR; ++j) {
             const int dm = dm0 + warp * DR + j;
+            int32_t *row = out + (size_t)dm * nout + t0 + quad_sample(lane);
 #pragma unroll
-            for (int i = 0; i < TI; ++i) {
-                const int64_t t = t0 + 4 * lane + 128 * (i / 4) + i % 4;
-                if (dm < a.ndm && t < nout) {
-                    const long long v = bs.at(j, i / 4, i % 4);
-                    out[(size_t)dm * nout + t] = (int32_t)v;
-                    n++; s += v; q += (unsigned long long)(v * v);
-                }
+            for (int i = 0; i < TI / 4; ++i) {
+                uint32_t v[4];
+                bs.at(j, i, lane, v);
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (dm < a.ndm && 128 * i + 32 * k < left) {
+                        row[128 * i + 32 * k] = (int32_t)v[k];
+                        n++; s += v[k]; q += (unsigned long long)v[k] * v[k];
+                    }
             }
         }
         block_stat_i(n, s, q, reinterpret_cast<StatI *>(a.partials) + lin);

@@ -164,12 +164,17 @@ __global__ void __launch_bounds__(NW * 32, 3) sub_kernel(SubLaunch a)
     if (!ok) return;
 
     // this lane's sample i of the tile
-    auto sample = [&](int i) { return t0 + (kBytes ? 4 * lane + 128 * (i / 4) + i % 4 : lane + 32 * i); };
+    auto sample = [&](int i) { return t0 + (kBytes ? quad_sample(lane) : lane) + 32 * i; };
     if constexpr (kBytes) {
 #pragma unroll
         for (int j = 0; j < DR; ++j)
 #pragma unroll
-            for (int i = 0; i < TI; ++i) acc[j][i] = (float)bs.at(j, i / 4, i % 4);   // exact: below 2^24
+            for (int i = 0; i < TI / 4; ++i) {
+                uint32_t v[4];
+                bs.at(j, i, lane, v);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) acc[j][4 * i + k] = (float)v[k];   // exact: below 2^24
+            }
     }
     const int64_t nout = a.nout;
     if constexpr (kInt) {
