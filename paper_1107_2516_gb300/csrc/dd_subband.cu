@@ -312,8 +312,12 @@ static int finish_stage(SubStage &st, long long need, size_t eb, size_t optin)
     // a block sums few channels (32 in the usual plans): 4 a stage, so that it
     // starts on the first while the others land (stage 2 of the LOFAR-like
     // plan 9.6 ms with 16 or 8 a stage, 8.2 with 4, which also lets a fourth
-    // block share the SM; stage 1 the same)
-    st.ch = (int)std::min<size_t>(4, budget / (kStages * per_ch));
+    // block share the SM; stage 1 the same).  Bytes, summed four channels at a
+    // time from rows a quarter as long: as many as fit (1024 channels in 32
+    // subbands, 2000 trials x 240 000 samples: stage 1 3.51 ms with 4, 2.98 with 8,
+    // 2.78 with 16; 96 in 2, 300 x 5000: 28.8, 24.3, 21.5 us, and 24.6 us with 16
+    // a stage and one byte a load)
+    st.ch = (int)std::min<size_t>(eb == 1 ? 16 : 4, budget / (kStages * per_ch));
     if (st.ch < 1) return set_error(DD_ERR_ARG, "subband rows too long for shared memory (%d samples)", st.rs);
     st.bar_off = (int)(((size_t)kStages * st.ch * per_ch + 15) / 16 * 16);
     st.smem = (size_t)st.bar_off + kStages * sizeof(uint64_t);
