@@ -200,8 +200,19 @@ DD_API int dd_process_host(dd_plan *plan, const void *in_host, int64_t in_pitch,
  * this plan. */
 DD_API int dd_plan_set_kernel(dd_plan *plan, int32_t kernel);
 
-/* Kernel that dd_execute will launch for this plan (1 to 5, see above). */
+/* Kernel selected for this plan (1 to 5, see above).  It says in which order a
+ * floating-point sum is formed; dd_plan_get_launch says what a launch runs
+ * (the finer shape of kernel 3 for few blocks, another kernel for rows that do
+ * not start on 16-byte boundaries). */
 DD_API int dd_plan_get_kernel(const dd_plan *plan, int32_t *kernel);
+
+/* What dd_execute launches for input rows at in_dev, in_pitch elements apart
+ * (the address is not read): the kernel (1 to 5), its configuration
+ * (dd_plan_set_tile's index; 13 = kernel 3's finer shape, which only the
+ * library chooses; -1 for kernel 1) and a block's DM trials and samples (any
+ * pointer may be NULL). */
+DD_API int dd_plan_get_launch(const dd_plan *plan, const void *in_dev, int64_t in_pitch, int32_t *kernel,
+                              int32_t *config, int32_t *trials_per_block, int32_t *samples_per_block);
 
 /* Autotuner for the tiled kernels: runs the plan on the caller's buffers
  * once per compiled tile configuration of kernels 2, 3 and 5 (0-6, 9-12,
@@ -231,7 +242,8 @@ DD_API int dd_plan_autotune(dd_plan *plan, const void *in_dev, int64_t in_pitch,
  * together.  DD_ERR_ARG if the configuration cannot run this plan. */
 DD_API int dd_plan_set_tile(dd_plan *plan, int32_t config, int32_t raster_group);
 
-/* Current tiled-kernel choice: configuration index, raster group, samples
+/* The plan's selected configuration (a launch may run another one:
+ * dd_plan_get_launch): configuration index, raster group, samples
  * per thread (kernel 2) or per lane (kernels 3-5) and warps per block (any
  * pointer may be NULL).  DD_ERR_ARG if the tiled kernels cannot run this
  * plan. */
@@ -450,7 +462,7 @@ DD_API int dd_server_beam_info(dd_server *server, int32_t beam, int64_t *maxshif
 DD_API int dd_server_set_autotune(dd_server *server, int32_t on);
 
 /* The kernel (dd_plan_get_kernel) and tile configuration (dd_plan_get_tile;
- * -1 for kernel 1) a beam runs; either pointer may be NULL. */
+ * -1 for kernel 1) selected for a beam; either pointer may be NULL. */
 DD_API int dd_server_beam_kernel(dd_server *server, int32_t beam, int32_t *kernel, int32_t *config);
 
 /* The host-side schedule the server follows for one beam, computed alone

@@ -361,6 +361,20 @@ int dd_plan_get_kernel(const dd_plan *plan, int32_t *kernel)
     return DD_OK;
 }
 
+int dd_plan_get_launch(const dd_plan *plan, const void *in_dev, int64_t in_pitch, int32_t *kernel, int32_t *config,
+                       int32_t *trials_per_block, int32_t *samples_per_block)
+{
+    if (!plan) return set_error(DD_ERR_ARG, "plan is NULL");
+    if (!in_dev || in_pitch < plan->nsamp_in) return set_error(DD_ERR_ARG, "bad input rows");
+    int k = 1, c = -1, t = kGenDms, n = kGenTile;
+    if (plan->kernel == 2) fast_launch_info(plan, in_dev, in_pitch, &k, &c, &t, &n);
+    if (kernel) *kernel = k;
+    if (config) *config = c;
+    if (trials_per_block) *trials_per_block = t;
+    if (samples_per_block) *samples_per_block = n;
+    return DD_OK;
+}
+
 int dd_plan_autotune(dd_plan *plan, const void *in_dev, int64_t in_pitch, void *out_dev, void *stream)
 {
     if (!plan) return set_error(DD_ERR_ARG, "plan is NULL");

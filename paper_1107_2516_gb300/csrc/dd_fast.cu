@@ -936,31 +936,63 @@ static int fast_run(dd_plan *p, int k, int dgroup, const void *in, int64_t pitch
     return DD_OK;
 }
 
+// Trials and samples of a block of configuration k (kFiner: kLaneSmall).
+constexpr int kFiner = kNumAllCfg;
+static void cfg_block(const FastPlan *f, int k, int *trials, int *samples)
+{
+    if (k == kFiner) { *trials = kLaneSmall.dr * kLaneSmall.nw; *samples = 32 * kLaneSmall.ti; }
+    else if (k >= kShareBeg) { const ShareShape &s = kShareCfg[k - kShareBeg]; *trials = s.dr * s.nw; *samples = 32 * s.ti; }
+    else if (k >= kLaneEnd) { *trials = kTmemCfg[k - kLaneEnd].dbw * f->tm[k - kLaneEnd].nw; *samples = 32 * f->tm[k - kLaneEnd].n; }
+    else if (k >= kNumFastCfg) { const LaneShape &l = kLaneCfg[k - kNumFastCfg]; *trials = l.dr * l.nw; *samples = 32 * l.ti; }
+    else { *trials = kDR * f->cfg[k].nw; *samples = 32 * f->cfg[k].tr; }
+}
+
+// What dd_execute launches for rows that start at `in`, `pitch` elements apart:
+// a configuration, kFiner, or -1 for the generic kernel.
+// Bulk copies need 16-byte aligned rows; for other rows the warp-specialised
+// kernel 5 and kernel 3 (plans whose tables kernel 5 does not take) stage
+// whole units around them, and where neither fits the generic kernel runs:
+// 200 channels x 150001 samples, 301 trials: 3.77 ms on the generic kernel,
+// 0.61 ms on kernel 5; 64 channels, 41 trials x 150001 samples: 166 us on
+// the generic kernel, 86 us on kernel 3 (float16 138 and 87, uint8 123 and
+// 83), x 8191 samples in its finer shape 54 and 13 us (uint8 48 and 11); 1024
+// channels, 64 trials x 8191 samples: 256 us on kernel 5, 103 us in the finer
+// shape (uint8 182 and 95).
+static int route(const dd_plan *p, const FastPlan *f, const void *in, int64_t pitch)
+{
+    const bool finer = f->small.ok && !f->forced && few_blocks(p, f);
+    int k = -1;
+    if (rows_aligned(f, in, pitch)) k = finer ? kFiner : f->active;
+    else if ((uintptr_t)in % in_elem_bytes(p->dtype)) return -1;
+    else if (finer && f->small.ch_any) k = kFiner;
+    else if (f->active >= kShareBeg && f->sh[kShareWs].ok && f->sh[kShareWs].ns_any) k = kShareBeg + kShareWs;
+    else if (f->active >= kNumFastCfg && f->active < kLaneEnd && f->lane[kLaneAny].ok && f->lane[kLaneAny].ch_any)
+        k = kNumFastCfg + kLaneAny;
+    if (k < 0) return -1;
+    int trials, samples;
+    cfg_block(f, k, &trials, &samples);
+    const int64_t blocks = ((p->nsamp_out + samples - 1) / samples) * ((p->ndm + trials - 1) / trials);
+    return blocks > INT32_MAX ? -1 : k;
+}
+
 int fast_execute(dd_plan *p, const void *in, int64_t pitch, void *out, cudaStream_t s)
 {
     FastPlan *f = static_cast<FastPlan *>(p->fast);
     if (!f) return set_error(DD_ERR_ARG, "kernel 2 unavailable for this plan");
-    // Bulk copies need 16-byte aligned rows; for other rows the warp-specialised
-    // kernel 5 and kernel 3 (plans whose tables kernel 5 does not take) stage
-    // whole units around them, and where neither fits the generic kernel runs:
-    // 200 channels x 150001 samples, 301 trials: 3.77 ms on the generic kernel,
-    // 0.61 ms on kernel 5; 64 channels, 41 trials x 150001 samples: 166 us on
-    // the generic kernel, 86 us on kernel 3 (float16 138 and 87, uint8 123 and
-    // 83), x 8191 samples in its finer shape 54 and 13 us (uint8 48 and 11); 1024
-    // channels, 64 trials x 8191 samples: 256 us on kernel 5, 103 us in the finer
-    // shape (uint8 182 and 95).
-    if (!rows_aligned(f, in, pitch)) {
-        const bool whole = (uintptr_t)in % in_elem_bytes(p->dtype) == 0;
-        if (whole && f->small.ok && f->small.ch_any && !f->forced && few_blocks(p, f))
-            return lane_run(p, -1, f->dgroup, in, pitch, out, s);
-        if (whole && f->active >= kShareBeg && f->sh[kShareWs].ok && f->sh[kShareWs].ns_any)
-            return fast_run(p, kShareBeg + kShareWs, f->dgroup, in, pitch, out, s);
-        if (whole && f->active >= kNumFastCfg && f->active < kLaneEnd && f->lane[kLaneAny].ok && f->lane[kLaneAny].ch_any)
-            return lane_run(p, kLaneAny, f->dgroup, in, pitch, out, s);
-        return generic_execute(p, in, pitch, out, s);
-    }
-    if (f->small.ok && !f->forced && few_blocks(p, f)) return lane_run(p, -1, f->dgroup, in, pitch, out, s);
-    return fast_run(p, f->active, f->dgroup, in, pitch, out, s);
+    const int k = route(p, f, in, pitch);
+    if (k < 0) return generic_execute(p, in, pitch, out, s);
+    return k == kFiner ? lane_run(p, -1, f->dgroup, in, pitch, out, s) : fast_run(p, k, f->dgroup, in, pitch, out, s);
+}
+
+void fast_launch_info(const dd_plan *p, const void *in, int64_t pitch, int *kernel, int *cfg, int *trials, int *samples)
+{
+    const FastPlan *f = static_cast<const FastPlan *>(p->fast);
+    const int k = f ? route(p, f, in, pitch) : -1;
+    *kernel = 1; *cfg = -1; *trials = kGenDms; *samples = kGenTile;
+    if (k < 0) return;
+    *cfg = k;
+    *kernel = k == kFiner ? 3 : k >= kShareBeg ? 5 : k >= kLaneEnd ? 4 : k >= kNumFastCfg ? 3 : 2;
+    cfg_block(f, k, trials, samples);
 }
 
 // Schedule of the pipelined host path for nsamp_out outputs in tiles of
@@ -993,7 +1025,7 @@ int fast_execute_host(dd_plan *p, const void *in_host, int64_t pitch, void *in_d
 {
     FastPlan *f = static_cast<FastPlan *>(p->fast);
     if (!f || ((uintptr_t)in_dev & 15u) || (pitch % f->al)) return kNotPipelined;
-    if (f->small.ok && !f->forced && few_blocks(p, f)) return kNotPipelined;   // one small launch
+    if (route(p, f, in_dev, pitch) == kFiner) return kNotPipelined;   // one small launch
     const int k = f->active;
     int tile, nblk;
     int64_t reach;

@@ -163,6 +163,8 @@ int fast_autotune(dd_plan *p, const void *in, int64_t pitch, void *out, cudaStre
 int fast_set_tile(dd_plan *p, int cfg, int dgroup);
 int fast_get_tile(const dd_plan *p, int *cfg, int *dgroup, int *tr, int *nw);
 int fast_kernel_id(const dd_plan *p);
+// kernel, configuration and block of the launch that dd_execute makes for these rows
+void fast_launch_info(const dd_plan *p, const void *in, int64_t pitch, int *kernel, int *cfg, int *trials, int *samples);
 void fast_unforce(dd_plan *p);     // the active shape counts as the default again
 
 }  // namespace dd

@@ -27,7 +27,7 @@ assert CANDIDATE_DTYPE.itemsize == 32
 # Names of every function declared in include/dd.h.
 EXPORTS = ("dd_plan_create", "dd_plan_destroy", "dd_plan_info", "dd_execute", "dd_search",
            "dd_last_stats", "dd_process_host", "dd_plan_set_kernel", "dd_plan_get_kernel",
-           "dd_plan_autotune", "dd_plan_set_tile", "dd_plan_get_tile",
+           "dd_plan_autotune", "dd_plan_set_tile", "dd_plan_get_tile", "dd_plan_get_launch",
            "dd_stats_f32_noalloc", "dd_last_error", "dd_version",
            "dd_batch_create", "dd_batch_destroy", "dd_batch_execute", "dd_batch_capture",
            "dd_batch_launch", "dd_batch_results", "dd_batch_autotune", "dd_batch_info", "dd_batch_set_config", "dd_batch_beam_config",
@@ -119,6 +119,7 @@ def load(path: Optional[str] = None):
             "dd_server_candidates": (C.c_int, [vp, i32, i64, vp, i64, P64]),
             "dd_server_beam_info": (C.c_int, [vp, i32, P64, P64, P64, C.POINTER(vp), P64]),
             "dd_server_memory": (C.c_int, [vp, P64, P64]),
+            "dd_plan_get_launch": (C.c_int, [vp, vp, i64] + [C.POINTER(i32)] * 4),
             "dd_plan_get_tile": (C.c_int, [vp, C.POINTER(i32), C.POINTER(i32), C.POINTER(i32),
                                            C.POINTER(i32)]),
             "dd_subband_plan_create": (C.c_int, [i32, f64, f64, f64, vp, i32, i32, i32, vp, i32, f64,
@@ -274,6 +275,13 @@ def dd_plan_get_tile(plan: int):
     """(config, raster_group, samples_per_thread, warps_per_block) of kernel 2."""
     v = [C.c_int32() for _ in range(4)]
     _check(load().dd_plan_get_tile(plan, *[C.byref(x) for x in v]))
+    return tuple(int(x.value) for x in v)
+
+
+def dd_plan_get_launch(plan: int, in_dev, in_pitch: int):
+    """(kernel, configuration, DM trials, samples per block) that dd_execute launches for these rows."""
+    v = [C.c_int32() for _ in range(4)]
+    _check(load().dd_plan_get_launch(plan, _ptr(in_dev), int(in_pitch), *[C.byref(x) for x in v]))
     return tuple(int(x.value) for x in v)
 
 
@@ -619,6 +627,10 @@ class Plan:
     @property
     def tile(self):
         return dd_plan_get_tile(self.handle)
+
+    def launch(self, in_dev, in_pitch):
+        """(kernel, configuration, DM trials, samples per block) execute runs for these rows."""
+        return dd_plan_get_launch(self.handle, in_dev, in_pitch)
 
     @property
     def kernel(self):

@@ -1,0 +1,74 @@
+"""What a launch runs (dd_plan_get_launch) against what the plan has selected:
+the finer shape of kernel 3 for few blocks, other kernels for rows that start
+anywhere, the caller's choice."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+import paper_1107_2516_gb300 as dd  # noqa: E402
+from test_share_ws_tables import CASES, TYPE  # noqa: E402
+
+FINER = (3, 13, 16, 128)
+WS = (5, 12, 64, 512)
+AL = {"f32": 4, "u8": 16, "f16": 8}
+
+
+@pytest.mark.parametrize("dtype", ["f32", "u8", "f16"])
+@pytest.mark.parametrize("case", range(len(CASES)))
+def test_few_blocks_of_a_kernel_5_plan(case, dtype):
+    nch, fch1, foff, ts, dms, nsamp, _ = CASES[case]
+    plan = dd.Plan(nch, fch1, foff, ts, dms, [1], 6.0, TYPE[dtype], nsamp)
+    pitch = -(-nsamp // AL[dtype]) * AL[dtype]
+    buf = torch.zeros((nch + 1) * (pitch + 16) * 4, dtype=torch.uint8, device="cuda").data_ptr()
+    eb = 16 // AL[dtype]
+    # float sums of 8-channel subbands (cases 2 and 3) have no finer shape
+    own = WS if dtype != "u8" and case in (2, 3) else FINER
+    assert plan.kernel == 5 and plan.tile[0] == 12
+    assert plan.launch(buf, pitch) == own
+    assert plan.launch(buf, pitch + 1) == plan.launch(buf + eb, pitch) == own
+    if eb > 1:
+        assert plan.launch(buf + 1, pitch) == (1, -1, 16, 512)       # not on an element
+    plan.set_tile(12, 8)
+    assert plan.launch(buf, pitch) == plan.launch(buf, pitch + 1) == WS
+    plan.set_tile(10, 8)
+    assert plan.launch(buf, pitch) == (5, 10, 32, 256) and plan.launch(buf, pitch + 1) == WS
+    plan.set_kernel(1)
+    assert plan.kernel == 1 and plan.launch(buf, pitch) == (1, -1, 16, 512)
+    plan.set_kernel(2)
+    assert plan.launch(buf, pitch)[:2] == (2, 0) and plan.launch(buf, pitch + 1)[0] == 1
+    plan.set_kernel(5)
+    assert plan.launch(buf, pitch) == WS
+    plan.set_kernel(0)
+    assert plan.launch(buf, pitch) == own
+    plan.close()
+
+
+def test_blocks_for_every_sm():
+    # as many blocks as SMs: kernel 3's own shape; more: kernel 5's; aligned rows or not
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for nch, step, want in ((65, 0.1, (3, 5, 32, 512)), (64, 0.01, WS)):
+        dms = [step * i for i in range(32)]
+        p0 = dd.Plan(nch, 150.0, -0.39, 327.68e-6, dms, [1], 6.0, dd.DD_F32, 1 << 17)
+        m = p0.maxshift
+        p0.close()
+        for tiles in (16, sms - 1, sms, sms + 1):
+            nsamp = 512 * tiles + m
+            plan = dd.Plan(nch, 150.0, -0.39, 327.68e-6, dms, [1], 6.0, dd.DD_F32, nsamp)
+            pitch = (nsamp + 3) // 4 * 4
+            x = torch.zeros(nch * (pitch + 1), device="cuda")
+            if want[0] == 3 and tiles < sms:
+                assert plan.launch(x, pitch) == plan.launch(x, pitch + 1) == FINER
+            elif tiles > sms or want[0] == 3:
+                assert plan.launch(x, pitch) == plan.launch(x, pitch + 1) == want
+            plan.close()
+
+
+def test_arguments():
+    plan = dd.Plan(4, 150.0, -0.1, 1e-3, [0.0], [1], 6.0, dd.DD_F32, 1000)
+    with pytest.raises(dd.DDError):
+        plan.launch(0, 1000)
+    with pytest.raises(dd.DDError):
+        plan.launch(16, 999)
+    plan.close()
