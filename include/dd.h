@@ -216,7 +216,8 @@ DD_API int dd_plan_get_launch(const dd_plan *plan, const void *in_dev, int64_t i
 
 /* Autotuner for the tiled kernels: runs the plan on the caller's buffers
  * once per compiled tile configuration of kernels 2, 3 and 5 (0-6, 9-12,
- * see dd_plan_set_tile) and raster group, times each with CUDA events on
+ * see dd_plan_set_tile; and kernel 3's finer shape, if the plan's launches have
+ * few blocks) and raster group, times each with CUDA events on
  * `stream`, keeps the fastest for this plan and caches the choice
  * process-wide for plans of the same shape.  Kernel 4 is not timed (slower on
  * every plan measured); dd_plan_set_kernel(plan, 4) selects it.  Writes

@@ -69,6 +69,7 @@ struct ShareCfgData {
 constexpr int kLaneEnd = kNumFastCfg + kNumLaneCfg;
 constexpr int kShareBeg = kLaneEnd + kNumTmemCfg;
 constexpr int kNumAllCfg = kShareBeg + kNumShareCfg;
+constexpr int kFiner = kNumAllCfg;   // kLaneSmall, beside the configurations that a caller can choose
 
 constexpr int kHostChunks = 8;   // input column chunks of the pipelined host path
 
@@ -77,6 +78,7 @@ struct FastPlan {
     LaneCfgData lane[kNumLaneCfg];
     LaneCfgData small;           // kLaneSmall, built for plans whose default launch leaves SMs empty
     bool forced = false;         // the caller chose the shape: small launches run it too
+    int finer = -1;              // the autotuner's choice of `small` (1) or the active shape (0); -1: few_blocks decides
     TmemCfgData tm[kNumTmemCfg];
     ShareCfgData sh[kNumShareCfg];
     int active = -1;
@@ -771,8 +773,9 @@ int fast_configure(dd_plan *p)
     if (f->active < 0) { fast_release(p); return DD_OK; }   // tiled kernels unavailable
     std::lock_guard<std::mutex> g(g_tune_mu);
     auto it = g_tune_cache.find(tune_key(p));
-    if (it != g_tune_cache.end() && cfg_ok(f, it->second.first)) {
-        f->active = it->second.first;
+    if (it != g_tune_cache.end() && (it->second.first == kFiner ? f->small.ok : cfg_ok(f, it->second.first))) {
+        f->finer = it->second.first == kFiner;
+        if (!f->finer) f->active = it->second.first;
         f->dgroup = it->second.second;
     }
     return DD_OK;
@@ -937,7 +940,6 @@ static int fast_run(dd_plan *p, int k, int dgroup, const void *in, int64_t pitch
 }
 
 // Trials and samples of a block of configuration k (kFiner: kLaneSmall).
-constexpr int kFiner = kNumAllCfg;
 static void cfg_block(const FastPlan *f, int k, int *trials, int *samples)
 {
     if (k == kFiner) { *trials = kLaneSmall.dr * kLaneSmall.nw; *samples = 32 * kLaneSmall.ti; }
@@ -960,7 +962,7 @@ static void cfg_block(const FastPlan *f, int k, int *trials, int *samples)
 // shape (uint8 182 and 95).
 static int route(const dd_plan *p, const FastPlan *f, const void *in, int64_t pitch)
 {
-    const bool finer = f->small.ok && !f->forced && few_blocks(p, f);
+    const bool finer = f->small.ok && !f->forced && (f->finer < 0 ? few_blocks(p, f) : f->finer == 1);
     int k = -1;
     if (rows_aligned(f, in, pitch)) k = finer ? kFiner : f->active;
     else if ((uintptr_t)in % in_elem_bytes(p->dtype)) return -1;
@@ -1087,24 +1089,31 @@ int fast_autotune(dd_plan *p, const void *in, int64_t pitch, void *out, cudaStre
     if (cudaEventCreate(&e0) != cudaSuccess) return set_error(DD_ERR_CUDA, "cudaEventCreate");
     if (cudaEventCreate(&e1) != cudaSuccess) { cudaEventDestroy(e0); return set_error(DD_ERR_CUDA, "cudaEventCreate"); }
     float best = 1e30f;
-    int bk = f->active, bg = f->dgroup, rc = DD_OK;
+    const int before = f->active;
+    int bk = before, bg = f->dgroup, rc = DD_OK;
+    f->active = first_cfg(f);    // the finer shape sums in this kernel's order
     // largest raster group first: on a tie (within 0.5%) it keeps the least DRAM
     // traffic (64: every DM block of the usual plans in one group, each time
     // tile's blocks together)
     const int groups[] = {64, 16, 8, 4};
+    // the finer shape (what the launches of a plan that has it run untimed), then
     // kernels 5, 3 and 2, each in its order of measured speed, so that a tie
-    // keeps the earlier one (kernel 5's warp-specialised 64-trial shape first, then the 48-trial one: fewest input
-    // re-reads); kernel 4 (slower on every plan measured) runs only on request
-    static const int order[] = {kShareBeg + 3, kShareBeg + 2, kShareBeg + 0, kShareBeg + 1, kNumFastCfg + 2,
+    // keeps the earlier one (kernel 5's warp-specialised 64-trial shape first,
+    // then the 48-trial one: fewest input re-reads); kernel 4 (slower on every
+    // plan measured) runs only on request
+    static const int order[] = {kFiner, kShareBeg + 3, kShareBeg + 2, kShareBeg + 0, kShareBeg + 1, kNumFastCfg + 2,
                                 kNumFastCfg + 0, kNumFastCfg + 3, kNumFastCfg + 1, 1, 0, 2};
-    static_assert(sizeof(order) / sizeof(order[0]) == kNumAllCfg - kNumTmemCfg, "every timed configuration once");
+    static_assert(sizeof(order) / sizeof(order[0]) == kNumAllCfg - kNumTmemCfg + 1, "every timed configuration once");
     for (int k : order) {
         if (rc != DD_OK) break;
-        if (!cfg_ok(f, k)) continue;
-        rc = fast_run(p, k, 8, in, pitch, out, s);             // warm-up (caches, clocks)
+        if (k == kFiner ? !f->small.ok : !cfg_ok(f, k)) continue;
+        auto run = [&](int g) {
+            return k == kFiner ? lane_run(p, -1, g, in, pitch, out, s) : fast_run(p, k, g, in, pitch, out, s);
+        };
+        rc = run(8);                                           // warm-up (caches, clocks)
         for (int gi = 0; gi < 4 && rc == DD_OK; ++gi) {
             cudaEventRecord(e0, s);
-            rc = fast_run(p, k, groups[gi], in, pitch, out, s);
+            rc = run(groups[gi]);
             cudaEventRecord(e1, s);
             if (rc) break;
             if (cudaEventSynchronize(e1) != cudaSuccess) { rc = set_error(DD_ERR_CUDA, "autotune sync"); break; }
@@ -1116,11 +1125,12 @@ int fast_autotune(dd_plan *p, const void *in, int64_t pitch, void *out, cudaStre
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (rc) return rc;
-    rc = fast_error(p, s);
-    if (rc) return rc;
-    f->active = bk;
+    if (rc == DD_OK) rc = fast_error(p, s);
+    if (rc) { f->active = before; return rc; }
+    f->finer = bk == kFiner;
+    if (bk != kFiner) f->active = bk;
     f->dgroup = bg;
+    f->forced = false;
     std::lock_guard<std::mutex> g(g_tune_mu);
     g_tune_cache[tune_key(p)] = {bk, bg};
     return DD_OK;
@@ -1136,6 +1146,7 @@ int fast_set_tile(dd_plan *p, int cfg, int dgroup)
     f->active = cfg;
     f->dgroup = dgroup;
     f->forced = true;
+    f->finer = -1;
     return DD_OK;
 }
 

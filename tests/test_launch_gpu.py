@@ -72,3 +72,40 @@ def test_arguments():
     with pytest.raises(dd.DDError):
         plan.launch(16, 999)
     plan.close()
+
+
+def test_the_autotuners_choice_is_what_runs():
+    # 1024 channels, 128 trials x 16384 samples of float16: 64 blocks of kernel 5's shape, which leave
+    # SMs empty and are still faster than the finer shape by 8%: the tuner keeps a shape that it timed as faster
+    nch, foff, ts, dms = 1024, -12.0 / 1024, 327.68e-6, [0.05 * i for i in range(128)]
+    p0 = dd.Plan(nch, 150.0, foff, ts, dms, [1], 6.0, dd.DD_F16, 1 << 16)
+    nsamp = 16384 + p0.maxshift
+    p0.close()
+    pitch = -(-nsamp // 8) * 8
+    x = torch.zeros(nch * pitch, dtype=torch.float16, device="cuda")
+    plan = dd.Plan(nch, 150.0, foff, ts, dms, [1], 6.0, dd.DD_F16, nsamp)
+    out = torch.empty(len(dms) * plan.nsamp_out, device="cuda")
+    plan.autotune(x, pitch, out)
+    assert plan.launch(x, pitch)[1] == plan.tile[0] != 13
+    again = dd.Plan(nch, 150.0, foff, ts, dms, [1], 6.0, dd.DD_F16, nsamp)        # starts from the cached choice
+    assert again.launch(x, pitch) == plan.launch(x, pitch)
+    again.close()
+    plan.close()
+
+
+def test_the_finer_shape_is_timed_too():
+    # 26 blocks of kernel 3's shape, nearly three times slower than the finer one: the tuner keeps that, also
+    # after another shape was chosen, and plans of the same shape start from it
+    args = (128, 150.0, -0.1953125, 327.68e-6, [0.1 * i for i in range(64)], [1], 6.0, dd.DD_F32, 8192)
+    plan = dd.Plan(*args)
+    x = torch.zeros(128 * 8192, device="cuda")
+    out = torch.empty(64 * plan.nsamp_out, device="cuda")
+    plan.set_tile(4, 8)
+    plan.autotune(x, 8192, out)
+    assert plan.launch(x, 8192) == FINER and plan.kernel == 3
+    again = dd.Plan(*args)
+    assert again.launch(x, 8192) == FINER and again.tile == plan.tile
+    again.set_tile(3, 8)
+    assert again.launch(x, 8192)[1] == 3
+    again.close()
+    plan.close()
