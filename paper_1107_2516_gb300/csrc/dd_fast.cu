@@ -57,6 +57,7 @@ struct ShareCfgData {
     int ns = 0;                  // input stages
     int64_t reach = 0;           // input columns a tile at t0 reads lie below t0 + reach
     size_t smem = 0;
+    double clocks = 0;           // warp-specialised shape: estimated clocks of its longest block (few_blocks)
     int bar_off_any = 0, ns_any = 0;   // the same for rows that start anywhere (ns_any 0: that form does not fit)
     size_t smem_any = 0;
     int32_t *d_rec = nullptr;    // [nblk][nsub][kLen] subband records
@@ -469,18 +470,38 @@ static void share_tables_ws(const int32_t *d, int D, int C, double foff, dd_dtyp
     }
 }
 
-// Estimated time of a subband's two stages, summed over the tables' records.
+// Estimated time of n subbands' two stages with `sums` partial sums together.
 // float: the shared-memory words that bound it, cs loads and a store per
 // partial sum and a load per trial and sample (1.33 to 1.38 clocks per 32 of
 // them measured with cs 4 and 8).  Packed: instructions bound it, measured 36
 // (cs 4) and 54 (cs 8) clocks per row of 128 sums and 330 per subband, 1050 at
 // least (stage 2).
-static double share_ws_cost(const ShareTables &T, int cs, bool packed)
+static double share_ws_cost(double n, double sums, int cs, bool packed)
 {
     const ShareShape &sh = kShareCfg[kShareWs];
-    const double n = (double)T.nblk * T.nsub, sums = (double)T.sums;
     if (packed) return std::max(1050.0 * n, 330.0 * n + sums / 128 * (18 + 4.5 * cs));
     return sums * (cs + 1) + n * sh.dr * sh.nw * 32 * sh.ti;
+}
+static double share_ws_cost(const ShareTables &T, int cs, bool packed)
+{
+    return share_ws_cost((double)T.nblk * T.nsub, (double)T.sums, cs, packed);
+}
+
+// The longest block's time in clocks, alone on its SM: each of its subbands as
+// above.  Packed sums take 1.2 (cs 8: 1.1) times their rows' clocks in one wave.
+static double share_ws_clocks(const ShareTables &T, int cs, bool packed)
+{
+    const ShareShape &sh = kShareCfg[kShareWs];
+    double most = 0;
+    for (int b = 0; b < T.nblk; ++b) {
+        double t = 0;
+        for (int s = 0; s < T.nsub; ++s) {
+            const int32_t *r = &T.rec[((size_t)b * T.nsub + s) * T.klen];
+            t += share_ws_cost(1, r[sh.dr * sh.nw] * (packed ? 4.0 : 1.0), cs, packed);   // its P entries (ShareRec::kE)
+        }
+        most = std::max(most, t);
+    }
+    return packed ? most * (cs == 8 ? 1.1 : 1.2) : most / 32 * 1.35;
 }
 
 // Shared memory of shape k with these tables, and the offsets in it.
@@ -568,6 +589,7 @@ static int build_share(const dd_plan *p, int k, ShareCfgData &c)
         // staged rows one 16-byte unit longer take rows that start anywhere
         const int rs = T.rs + (int)(16 / eb);
         c.ns_any = share_ws_stages(T, cs, rs, eb, p->smem_optin);
+        c.clocks = share_ws_clocks(T, cs, p->dtype == DD_U8);
         const ShareLayout u = share_layout(T, k, cs, rs, eb, c.ns_any);
         if (c.ns_any) { c.bar_off_any = (int)u.bar_off; c.smem_any = u.bytes; }
     }
@@ -711,32 +733,44 @@ static int first_cfg(const FastPlan *f)
 // finer shape kLaneSmall, with 8 or 16 times the blocks, is faster.  A block
 // alone on an SM is a chain of loads and adds over all channels.
 // Kernel 3 shapes: 64 trials x 6600 samples of 128 channels (26 blocks) 58 us,
-// 20 us with the finer shape; from one block per SM on the larger shapes'
-// fewer staged samples per sum count for more (512 blocks: 162 against 157 us).
-// Kernel 5 adds fewer words, so there the time decides: measured, one wave of
-// the warp-specialised shape takes 2300 clocks per subband (uint8 1650, of 8
-// channels 1.25 times that), the finer shape 157 per channel or 1.25 per 32
-// words and SM.  1024 channels, 64 trials x 8192 samples: 298 -> 113 us (uint8
-// 214 -> 87); 128 x 16384: 307 and 287 (216 and 234).
+// 20 us with the finer shape, 150 blocks 58 and 51 us; from one block per SM on
+// the larger shapes' fewer staged samples per sum count for more (512 blocks: 162
+// against 157 us).
+// Kernel 5's one-barrier shapes, up to one block per SM: 256 channels, 32 blocks 137
+// and 32 us (uint8 141 and 24), 128 blocks 124 and 78 us (uint8 131 and 62).
+// The warp-specialised shape adds fewer words, so there the time decides: a wave
+// takes its longest block's estimate and 26 000 clocks to fill and drain (uint8
+// 16 000); the finer shape 12 000 (8000) and, per channel and block on an SM, 80
+// clocks (float16 84, uint8 66), half of that for the warps whose trials do
+// not exist, but 157 (125) per channel at least.  1024 channels, 64 trials x 8192
+// samples: 252 and 99 us (float16 250 and 109, uint8 172 and 85); x 24576: 255 and
+// 247; 128 x 16384: 277 and 281 (float16 273 and 296, uint8 199 and 233), where
+// the wave stays.  Over 509 such launches (128 to 4096 channels, 8 to 200 trials,
+// each type) the choice is 0.1% from the faster one on average, 7% at worst.
 static bool few_blocks(const dd_plan *p, const FastPlan *f)
 {
     const int k = f->active;
-    auto blocks = [&](int ti, int db) {
-        return ((p->nsamp_out + 32 * ti - 1) / (32 * ti)) * (int64_t)((p->ndm + db - 1) / db);
-    };
+    const int64_t sms = p->sm_count;
+    auto tiles = [&](int ti) { return (p->nsamp_out + 32 * ti - 1) / (32 * ti); };
+    auto blocks = [&](int ti, int db) { return tiles(ti) * (int64_t)((p->ndm + db - 1) / db); };
     if (k >= kNumFastCfg && k < kLaneEnd) {
         const LaneShape &l = kLaneCfg[k - kNumFastCfg];
-        return blocks(l.ti, l.dr * l.nw) < p->sm_count;
+        return blocks(l.ti, l.dr * l.nw) < sms;
     }
     if (k < kShareBeg) return false;
     const ShareShape &sh = kShareCfg[k - kShareBeg];
     const ShareCfgData &c = f->sh[k - kShareBeg];
+    const bool u8 = p->dtype == DD_U8;
     // float sums of 8-channel subbands are rounded in another order: not to the bit
-    if (p->nchans % 4 || (c.cs == 8 && p->dtype != DD_U8) || blocks(sh.ti, sh.dr * sh.nw) > p->sm_count) return false;
-    const double wave = c.nsub * (p->dtype == DD_U8 ? 1650.0 : 2300.0) * (c.cs == 8 ? 1.25 : 1.0);
-    const int db = kLaneSmall.dr * kLaneSmall.nw, tile = 32 * kLaneSmall.ti;
-    const double words = (double)blocks(kLaneSmall.ti, db) * db * tile * p->nchans / 32;
-    return std::max(157.0 * p->nchans, 1.25 * words / p->sm_count) < wave;
+    if (p->nchans % 4 || (c.cs == 8 && !u8) || blocks(sh.ti, sh.dr * sh.nw) > sms) return false;
+    if (sh.pw == 0) return true;
+    auto per_sm = [&](int64_t n) { return (double)((n + sms - 1) / sms); };
+    const LaneShape &l = kLaneSmall;
+    const double n = 0.5 * per_sm(blocks(l.ti, l.dr * l.nw)) +
+                     0.5 * per_sm((tiles(l.ti) * ((p->ndm + l.dr - 1) / l.dr) + l.nw - 1) / l.nw);
+    const double fine = (u8 ? 8000 : 12000) +
+                        p->nchans * std::max(u8 ? 125.0 : 157.0, (u8 ? 66 : p->dtype == DD_F16 ? 84 : 80) * n);
+    return fine < (u8 ? 16000 : 26000) + c.clocks;
 }
 
 int fast_configure(dd_plan *p)

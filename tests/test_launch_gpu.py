@@ -109,3 +109,33 @@ def test_the_finer_shape_is_timed_too():
     assert again.launch(x, 8192)[1] == 3
     again.close()
     plan.close()
+
+
+@pytest.mark.parametrize("dtype,nout,want", [("f32", 8192, FINER), ("f16", 8192, FINER), ("u8", 8192, FINER),
+                                             ("f16", 2 * 16384, WS), ("u8", 2 * 16384, WS)])
+def test_the_estimate_keeps_the_faster_wave(dtype, nout, want):
+    # 1024 channels, 64 trials: 16 blocks of kernel 5's shape run 2 to 2.5 times longer than the finer
+    # one, 64 blocks (here in time; 128 x 16384 timed) 8% shorter for float16 and 15% for uint8
+    nch, foff, ts, dms = 1024, -12.0 / 1024, 327.68e-6, [0.05 * i for i in range(64)]
+    p0 = dd.Plan(nch, 150.0, foff, ts, dms, [1], 6.0, TYPE[dtype], 1 << 17)
+    nsamp = nout + p0.maxshift
+    p0.close()
+    plan = dd.Plan(nch, 150.0, foff, ts, dms, [1], 6.0, TYPE[dtype], nsamp)
+    assert plan.launch(1 << 20, -(-nsamp // 16) * 16) == want
+    plan.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "u8"])
+def test_one_barrier_shapes_leave_few_blocks_to_the_finer_one(dtype):
+    # delay patterns that only kernel 5's shapes of 48 or 32 trials take, up to one block per SM
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    nch, foff, ts, dms = 256, -12.0 / 256, 163.84e-6, [0.05 * i for i in range(64)]
+    p0 = dd.Plan(nch, 150.0, foff, ts, dms, [1], 6.0, TYPE[dtype], 1 << 17)
+    m = p0.maxshift
+    p0.close()
+    for tiles, few in ((16, True), (sms // 2, True), (sms // 2 + 1, False)):
+        nsamp = 512 * tiles + m
+        plan = dd.Plan(nch, 150.0, foff, ts, dms, [1], 6.0, TYPE[dtype], nsamp)
+        assert plan.tile[0] == 11
+        assert plan.launch(1 << 20, -(-nsamp // 16) * 16) == (FINER if few else (5, 11, 48, 512))
+        plan.close()
