@@ -305,9 +305,8 @@ DD_API int dd_batch_autotune(dd_batch *batch, const void *const *in_devs, const 
 DD_API int dd_host_chunk_schedule(int64_t nsamp_out, int64_t pitch, int32_t tile, int64_t reach,
                                   int64_t *col_end, int64_t *tile_end, int32_t *n);
 
-/* Kernel 5's tables for tile configuration `config` (9-12; 12 in the form with
- * 4-channel subbands and float sums, what it runs with is
- * dd_share_ws_tables') of a delay table
+/* Kernel 5's sums for tile configuration `config` (9-12; 12 in the form with
+ * 4-channel subbands and float sums) of a delay table
  * delays[ndm][nchans] (dd_plan_info's copy), computed on the host (no device
  * needed), for inspection and tests.  info[6] receives {1 if the shape can
  * run the table (at most 16 delay patterns per block and subband) else 0,
@@ -321,21 +320,34 @@ DD_API int dd_host_chunk_schedule(int64_t nsamp_out, int64_t pitch, int32_t tile
  * int32 [2][blocks][nchans]: the staged row starts relative to a tile's
  * first output sample, then the staged row lengths (the elements the block's
  * trials read, in 16-byte units; at most rs).  foff's sign picks the subband
- * reference channel (the highest frequency).  DD_ERR_ARG for another
- * configuration or too small a capacity. */
+ * reference channel (the highest frequency).  The sums are those a launch forms;
+ * their split over the warps at each record's end is this call's own (warp 0 with
+ * 70 or, configuration 12, 50 percent of another warp's rows): no kernel runs
+ * it, and whether the buffers fit an SM is not looked at.  What a launch runs
+ * with is dd_share_run_tables'.  DD_ERR_ARG for another configuration or too
+ * small a capacity. */
 DD_API int dd_share_tables(const int32_t *delays, int32_t ndm, int32_t nchans, double foff, int32_t dtype,
                            int32_t config, int32_t *info, int32_t *rec_out, int64_t rec_cap, int32_t *base_out,
                            int64_t base_cap);
 
-/* The tables that configuration 12 runs with (host only), for inspection and
- * tests: subbands of 4 or, where they move fewer shared-memory words, of 8
- * channels; for DD_U8 the partial sums are counted in quads of four and read
+/* The tables that configuration `config` (9-12) runs with, as a plan uploads them
+ * (host only), for inspection and tests; info[0] is 0 where it cannot run the
+ * table or its buffers do not fit.  Behind the patterns a record holds the first
+ * row of 32 sums (packed: quads) of each stage-1 warp, 9 words, and the pattern that
+ * row is in, 8 words.  Configuration 12 has subbands of 4 or, where they move
+ * fewer shared-memory words, of 8
+ * channels; for DD_U8 its partial sums are counted in quads of four and read
  * as pairs.  info[8] = dd_share_tables' six words, channels per subband, 1 if
  * packed.  Records as dd_share_tables' with info[6] offsets per pattern (each
  * pattern a whole number of 16-byte units); packed: pattern ends and starts in
  * quads, offsets such that quad e's first term is staged element offset + 4e,
  * a trial's index the word of its first pair (pairs from even sums in the
  * first half of pmax words, from odd sums in the second). */
+DD_API int dd_share_run_tables(const int32_t *delays, int32_t ndm, int32_t nchans, double foff, int32_t dtype,
+                               int32_t config, int32_t *info, int32_t *rec_out, int64_t rec_cap,
+                               int32_t *base_out, int64_t base_cap);
+
+/* dd_share_run_tables of configuration 12. */
 DD_API int dd_share_ws_tables(const int32_t *delays, int32_t ndm, int32_t nchans, double foff, int32_t dtype,
                               int32_t *info, int32_t *rec_out, int64_t rec_cap, int32_t *base_out,
                               int64_t base_cap);

@@ -330,7 +330,7 @@ static void split_rows(const std::vector<int> &n, int nw, int *b)
 
 template <int DB, int CS = kShCS, bool kQuad = false>
 static void share_tables_db(const int32_t *delays, int D, int C, double foff, dd_dtype dtype, int k,
-                            ShareTables &T, int w0)
+                            ShareTables &T)
 {
     T = ShareTables();
     constexpr int NP = kShNP, U = kQuad ? 4 : 1;   // samples per P index
@@ -402,18 +402,14 @@ static void share_tables_db(const int32_t *delays, int D, int C, double foff, dd
                 rows += (W + 31) / 32;
             }
             prow[np] = rows;
-            // stage-1 split: warp w's first row and the pattern holding it.
-            // Warp 0 gets w0 percent of another warp's share of the rows, the
-            // others equal shares; packed sums: split_rows.
+            // stage-1 split: warp w's first row and the pattern holding it;
+            // equal shares of the rows, packed sums: split_rows.
             if (kQuad) {
                 nrow.resize(np);
                 for (int q = 0; q < np; ++q) nrow[q] = prow[q + 1] - prow[q];
                 split_rows(nrow, nw, t + R::kWarp);
             } else {
-                const long long tot = w0 + 100LL * (nw - 1);
-                t[R::kWarp] = 0;
-                for (int w = 1; w <= nw; ++w)
-                    t[R::kWarp + w] = (int)(((long long)rows * (w0 + 100LL * (w - 1)) + tot / 2) / tot);
+                for (int w = 0; w <= nw; ++w) t[R::kWarp + w] = (int)((2LL * rows * w + nw) / (2 * nw));
             }
             for (int w = 0; w < nw; ++w) {
                 const int r0 = t[R::kWarp + w];
@@ -444,13 +440,12 @@ static void share_tables_db(const int32_t *delays, int D, int C, double foff, dd
     T.ok = true;
 }
 
-static void share_tables(const int32_t *delays, int D, int C, double foff, dd_dtype dtype, int k, ShareTables &T,
-                         int w0 = 100)
+static void share_tables(const int32_t *delays, int D, int C, double foff, dd_dtype dtype, int k, ShareTables &T)
 {
     switch (kShareCfg[k].dr * kShareCfg[k].nw) {
-    case 32: share_tables_db<32>(delays, D, C, foff, dtype, k, T, w0); break;
-    case 48: share_tables_db<48>(delays, D, C, foff, dtype, k, T, w0); break;
-    case 64: share_tables_db<64>(delays, D, C, foff, dtype, k, T, w0); break;
+    case 32: share_tables_db<32>(delays, D, C, foff, dtype, k, T); break;
+    case 48: share_tables_db<48>(delays, D, C, foff, dtype, k, T); break;
+    case 64: share_tables_db<64>(delays, D, C, foff, dtype, k, T); break;
     default: T = ShareTables(); break;
     }
 }
@@ -461,12 +456,12 @@ static void share_tables_ws(const int32_t *d, int D, int C, double foff, dd_dtyp
     constexpr int k = kShareWs;
     static_assert(kShareCfg[k].dr * kShareCfg[k].nw == 64, "the warp-specialised shape's trials per block");
     if (dtype == DD_U8) {
-        if (cs == 8) share_tables_db<64, 8, true>(d, D, C, foff, dtype, k, T, 100);
-        else share_tables_db<64, 4, true>(d, D, C, foff, dtype, k, T, 100);
+        if (cs == 8) share_tables_db<64, 8, true>(d, D, C, foff, dtype, k, T);
+        else share_tables_db<64, 4, true>(d, D, C, foff, dtype, k, T);
     } else if (cs == 8) {
-        share_tables_db<64, 8>(d, D, C, foff, dtype, k, T, 100);
+        share_tables_db<64, 8>(d, D, C, foff, dtype, k, T);
     } else {
-        share_tables_db<64>(d, D, C, foff, dtype, k, T, 100);
+        share_tables_db<64>(d, D, C, foff, dtype, k, T);
     }
 }
 
@@ -563,23 +558,26 @@ static int share_ws_choose(const int32_t *d, int D, int C, double foff, dd_dtype
     return 8;
 }
 
+// The tables that shape k runs with; T.ok is false where it cannot run them.
+// Returns the channels per subband.
+static int share_run_tables(const int32_t *d, int D, int C, double foff, dd_dtype dtype, int k, size_t optin, ShareTables &T)
+{
+    if (kShareCfg[k].pw > 0) return share_ws_choose(d, D, C, foff, dtype, optin, T);
+    share_tables(d, D, C, foff, dtype, k, T);
+    if (T.ok) T.ok = share_fits(k, share_layout(T, k, kShCS, T.rs, in_elem_bytes(dtype), kShareCfg[k].ns).bytes, optin);
+    return kShCS;
+}
+
 static int build_share(const dd_plan *p, int k, ShareCfgData &c)
 {
     c = ShareCfgData();
     const ShareShape &sh = kShareCfg[k];
     const size_t eb = in_elem_bytes(p->dtype);
+    if (!share_regs_ok(k, p->dtype)) return DD_OK;
     ShareTables T;
-    int cs = kShCS;
-    if (sh.pw > 0) {
-        if (!share_regs_ok(k, p->dtype)) return DD_OK;
-        cs = share_ws_choose(p->delays.data(), p->ndm, p->nchans, p->foff, p->dtype, p->smem_optin, T);
-        if (!T.ok) return DD_OK;
-        c.ns = share_ws_stages(T, cs, T.rs, eb, p->smem_optin);
-    } else {
-        c.ns = sh.ns;
-        share_tables(p->delays.data(), p->ndm, p->nchans, p->foff, p->dtype, k, T);
-        if (!T.ok || !share_fits(k, share_layout(T, k, cs, T.rs, eb, c.ns).bytes, p->smem_optin)) return DD_OK;
-    }
+    const int cs = share_run_tables(p->delays.data(), p->ndm, p->nchans, p->foff, p->dtype, k, p->smem_optin, T);
+    if (!T.ok) return DD_OK;
+    c.ns = sh.pw > 0 ? share_ws_stages(T, cs, T.rs, eb, p->smem_optin) : sh.ns;
     const ShareLayout l = share_layout(T, k, cs, T.rs, eb, c.ns);
     c.reach = (int64_t)*std::max_element(T.base.begin(), T.base.begin() + (size_t)T.nblk * p->nchans) + T.rs;
     c.nblk = T.nblk; c.nsub = T.nsub; c.rs = T.rs; c.pmax = l.pmax; c.bar_off = (int)l.bar_off;
@@ -1539,16 +1537,9 @@ int dd_host_chunk_schedule(int64_t nsamp_out, int64_t pitch, int32_t tile, int64
     return DD_OK;
 }
 
-int dd_share_tables(const int32_t *delays, int32_t ndm, int32_t nchans, double foff, int32_t dtype,
-                    int32_t config, int32_t *info, int32_t *rec_out, int64_t rec_cap, int32_t *base_out,
-                    int64_t base_cap)
+static int copy_tables(const ShareTables &T, int32_t *info, int32_t *rec_out, int64_t rec_cap, int32_t *base_out,
+                       int64_t base_cap)
 {
-    if (!delays || !info || ndm < 1 || nchans < 1) return set_error(DD_ERR_ARG, "bad table arguments");
-    if (dtype != DD_F32 && dtype != DD_U8 && dtype != DD_F16) return set_error(DD_ERR_ARG, "bad dtype %d", dtype);
-    if (config < kShareBeg || config >= kShareBeg + kNumShareCfg)
-        return set_error(DD_ERR_ARG, "configuration %d is not a kernel 5 shape", config);
-    ShareTables T;
-    share_tables(delays, ndm, nchans, foff, (dd_dtype)dtype, config - kShareBeg, T, kShareCfg[config - kShareBeg].w0);
     info[0] = T.ok ? 1 : 0;
     info[1] = T.nblk; info[2] = T.nsub; info[3] = T.rs; info[4] = T.pmax; info[5] = T.klen;
     if (!T.ok) return DD_OK;
@@ -1563,26 +1554,59 @@ int dd_share_tables(const int32_t *delays, int32_t ndm, int32_t nchans, double f
     return DD_OK;
 }
 
-int dd_share_ws_tables(const int32_t *delays, int32_t ndm, int32_t nchans, double foff, int32_t dtype, int32_t *info,
-                       int32_t *rec_out, int64_t rec_cap, int32_t *base_out, int64_t base_cap)
+int dd_share_tables(const int32_t *delays, int32_t ndm, int32_t nchans, double foff, int32_t dtype,
+                    int32_t config, int32_t *info, int32_t *rec_out, int64_t rec_cap, int32_t *base_out,
+                    int64_t base_cap)
 {
     if (!delays || !info || ndm < 1 || nchans < 1) return set_error(DD_ERR_ARG, "bad table arguments");
     if (dtype != DD_F32 && dtype != DD_U8 && dtype != DD_F16) return set_error(DD_ERR_ARG, "bad dtype %d", dtype);
+    if (config < kShareBeg || config >= kShareBeg + kNumShareCfg)
+        return set_error(DD_ERR_ARG, "configuration %d is not a kernel 5 shape", config);
+    const int k = config - kShareBeg;
     ShareTables T;
-    const int cs = share_ws_choose(delays, ndm, nchans, foff, (dd_dtype)dtype, 227 * 1024, T);
-    info[0] = T.ok ? 1 : 0;
-    info[1] = T.nblk; info[2] = T.nsub; info[3] = T.rs; info[4] = T.pmax; info[5] = T.klen;
-    info[6] = cs; info[7] = dtype == DD_U8 ? 1 : 0;
-    if (!T.ok) return DD_OK;
-    if (rec_out) {
-        if (rec_cap < (int64_t)T.rec.size()) return set_error(DD_ERR_ARG, "record buffer too small");
-        memcpy(rec_out, T.rec.data(), T.rec.size() * 4);
+    share_tables(delays, ndm, nchans, foff, (dd_dtype)dtype, k, T);
+    if (T.ok) {
+        // this call's own stage-1 split: warp 0 with 70 (configuration 12: 50) percent of another warp's rows
+        const ShareShape &sh = kShareCfg[k];
+        const int nw = sh.pw > 0 ? sh.pw : sh.nw, w0 = sh.pw > 0 ? 50 : 70, tot = w0 + 100 * (nw - 1);
+        const int db = sh.dr * sh.nw;
+        using R = ShareRecDB<32>;       // the fields behind the trials do not depend on their number
+        for (size_t i = 0; i < T.rec.size(); i += T.klen) {
+            int32_t *t = &T.rec[i] + (db - 32);
+            auto pat = [&](int q, int field) { return t[R::kPat + q * R::kPatLen + field]; };
+            int np = 0;
+            while (pat(np, 0) != t[R::kE]) ++np;
+            const long long rows = pat(np, R::kPatRows) + (pat(np, 0) - pat(np, R::kPatStart) + 31) / 32;
+            for (int w = 1; w <= nw; ++w) t[R::kWarp + w] = (int)((rows * (w0 + 100 * (w - 1)) + tot / 2) / tot);
+            for (int w = 0; w < nw; ++w) {
+                int q = 0;
+                while (q < np && pat(q + 1, R::kPatRows) <= t[R::kWarp + w]) ++q;
+                t[R::kWarp + R::kMaxWarps + 1 + w] = q;
+            }
+        }
     }
-    if (base_out) {
-        if (base_cap < (int64_t)T.base.size()) return set_error(DD_ERR_ARG, "row-start buffer too small");
-        memcpy(base_out, T.base.data(), T.base.size() * 4);
-    }
-    return DD_OK;
+    return copy_tables(T, info, rec_out, rec_cap, base_out, base_cap);
+}
+
+int dd_share_run_tables(const int32_t *delays, int32_t ndm, int32_t nchans, double foff, int32_t dtype, int32_t config,
+                        int32_t *info, int32_t *rec_out, int64_t rec_cap, int32_t *base_out, int64_t base_cap)
+{
+    if (!delays || !info || ndm < 1 || nchans < 1) return set_error(DD_ERR_ARG, "bad table arguments");
+    if (dtype != DD_F32 && dtype != DD_U8 && dtype != DD_F16) return set_error(DD_ERR_ARG, "bad dtype %d", dtype);
+    if (config < kShareBeg || config >= kShareBeg + kNumShareCfg)
+        return set_error(DD_ERR_ARG, "configuration %d is not a kernel 5 shape", config);
+    const int k = config - kShareBeg;
+    ShareTables T;
+    info[6] = share_run_tables(delays, ndm, nchans, foff, (dd_dtype)dtype, k, 227 * 1024, T);
+    info[7] = kShareCfg[k].pw > 0 && dtype == DD_U8 ? 1 : 0;
+    return copy_tables(T, info, rec_out, rec_cap, base_out, base_cap);
+}
+
+int dd_share_ws_tables(const int32_t *delays, int32_t ndm, int32_t nchans, double foff, int32_t dtype, int32_t *info,
+                       int32_t *rec_out, int64_t rec_cap, int32_t *base_out, int64_t base_cap)
+{
+    return dd_share_run_tables(delays, ndm, nchans, foff, dtype, kShareBeg + kShareWs, info, rec_out, rec_cap, base_out,
+                               base_cap);
 }
 
 int dd_batch_create(dd_plan *const *plans, int32_t nplans, dd_batch **out)

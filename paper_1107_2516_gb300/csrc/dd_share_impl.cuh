@@ -114,7 +114,7 @@ __device__ __forceinline__ void share_raster(const ShareLaunch &a, int64_t lin, 
 // Stage 1 of one subband: P[e] for e < E (the patterns' sums end to end).
 // Each pattern's sums form rows of 32 consecutive e (the last one partial);
 // warp w takes the contiguous rows the record assigns it (the host splits
-// the R rows in order, warp 0 a smaller share), so a row's pattern (its fields) is
+// the R rows in order, equal shares), so a row's pattern (its fields) is
 // uniform in the warp and changes only at pattern ends, and lane l sums
 // element row_start + l of each of its rows: whole rows RPS at a time with
 // the pattern's offsets set up once (every load of a step issued before its
@@ -875,16 +875,13 @@ __global__ void __launch_bounds__((NW + PW + kWsStage) * 32, 1) share_ws_kernel(
 // warp, warps (stage-2 warps in the warp-specialised form), resident blocks
 // per SM the register budget targets, input stages (at most, in the
 // warp-specialised form), stage-1 warps (0: the one-barrier-per-subband
-// kernel, whose warps do both stages), partial-sum slots, stage-1 rows of warp
-// 0 in percent of another warp's in dd_share_tables' records (from the time
-// when its first thread issued all input copies; the kernels' own tables give
-// every warp an equal share)}.
+// kernel, whose warps do both stages), partial-sum slots}.
 constexpr int kShCS = 4, kShNP = 16;
-struct ShareShape { int ti, dr, nw, minb, ns, pw, pb, w0; };
+struct ShareShape { int ti, dr, nw, minb, ns, pw, pb; };
 constexpr int kNumShareCfg = 4;
 constexpr int kShareWs = 3;          // the warp-specialised shape
 constexpr ShareShape kShareCfg[kNumShareCfg] = {
-    {16, 8, 4, 3, 2, 0, 2, 70}, {8, 8, 4, 5, 2, 0, 2, 70}, {16, 8, 6, 2, 2, 0, 2, 70}, {16, 8, 8, 1, 6, 8, 3, 50}};
+    {16, 8, 4, 3, 2, 0, 2}, {8, 8, 4, 5, 2, 0, 2}, {16, 8, 6, 2, 2, 0, 2}, {16, 8, 8, 1, 6, 8, 3}};
 template <int DB>
 using ShareRecDB = ShareRec<kShCS, kShNP, DB>;
 

@@ -31,7 +31,7 @@ EXPORTS = ("dd_plan_create", "dd_plan_destroy", "dd_plan_info", "dd_execute", "d
            "dd_stats_f32_noalloc", "dd_last_error", "dd_version",
            "dd_batch_create", "dd_batch_destroy", "dd_batch_execute", "dd_batch_capture",
            "dd_batch_launch", "dd_batch_results", "dd_batch_autotune", "dd_batch_info", "dd_batch_set_config", "dd_batch_beam_config",
-           "dd_batch_set_launch_mode", "dd_batch_launch_mode", "dd_share_tables", "dd_share_ws_tables",
+           "dd_batch_set_launch_mode", "dd_batch_launch_mode", "dd_share_tables", "dd_share_ws_tables", "dd_share_run_tables",
            "dd_host_chunk_schedule",
            "dd_server_create", "dd_server_destroy", "dd_server_add_beam", "dd_server_remove_beam",
            "dd_server_submit", "dd_server_poll", "dd_server_candidates", "dd_server_beam_info",
@@ -108,6 +108,7 @@ def load(path: Optional[str] = None):
             "dd_batch_launch_mode": (C.c_int, [vp, C.POINTER(i32)]),
             "dd_share_tables": (C.c_int, [vp, i32, i32, f64, i32, i32, vp, vp, i64, vp, i64]),
             "dd_share_ws_tables": (C.c_int, [vp, i32, i32, f64, i32, vp, vp, i64, vp, i64]),
+            "dd_share_run_tables": (C.c_int, [vp, i32, i32, f64, i32, i32, vp, vp, i64, vp, i64]),
             "dd_host_chunk_schedule": (C.c_int, [i64, i64, i32, i64, vp, vp, C.POINTER(i32)]),
             "dd_server_create": (C.c_int, [i64, i32, i64, C.POINTER(vp)]),
             "dd_server_destroy": (C.c_int, [vp]),
@@ -404,22 +405,27 @@ def dd_share_tables(delays: np.ndarray, foff: float, dtype: int, config: int):
     return {"rec": rec, "base": base[0], "rlen": base[1], "rs": rs, "pmax": pmax, "klen": klen}
 
 
-def dd_share_ws_tables(delays: np.ndarray, foff: float, dtype: int):
-    """The tables configuration 12 runs with (host only): dd_share_tables' dict
+def dd_share_run_tables(delays: np.ndarray, foff: float, dtype: int, config: int):
+    """The tables configuration `config` runs with (host only): dd_share_tables' dict
     with the channels per subband (cs) and whether the sums are packed, or None."""
     d = np.ascontiguousarray(delays, dtype=np.int32)
     ndm, nch = d.shape
     info = np.zeros(8, np.int32)
-    _check(load().dd_share_ws_tables(_ptr(d), ndm, nch, float(foff), int(dtype), _ptr(info), None, 0, None, 0))
+    args = (_ptr(d), ndm, nch, float(foff), int(dtype), int(config), _ptr(info))
+    _check(load().dd_share_run_tables(*args, None, 0, None, 0))
     if not info[0]:
         return None
     nblk, nsub, rs, pmax, klen, cs, packed = (int(v) for v in info[1:])
     rec = np.empty((nblk, nsub, klen), np.int32)
     base = np.empty((2, nblk, nch), np.int32)
-    _check(load().dd_share_ws_tables(_ptr(d), ndm, nch, float(foff), int(dtype), _ptr(info), _ptr(rec), rec.size,
-                                     _ptr(base), base.size))
+    _check(load().dd_share_run_tables(*args, _ptr(rec), rec.size, _ptr(base), base.size))
     return {"rec": rec, "base": base[0], "rlen": base[1], "rs": rs, "pmax": pmax, "klen": klen, "cs": cs,
             "packed": bool(packed)}
+
+
+def dd_share_ws_tables(delays: np.ndarray, foff: float, dtype: int):
+    """dd_share_run_tables of configuration 12."""
+    return dd_share_run_tables(delays, foff, dtype, 12)
 
 
 def dd_batch_beam_config(batch: int, beam: int) -> int:
