@@ -148,6 +148,10 @@ DD_API int dd_execute(dd_plan *plan, const void *in_dev, int64_t in_pitch, void 
 DD_API int dd_search(dd_plan *plan, const void *out_dev, dd_candidate *cand_host,
               int64_t capacity, int64_t *n_found, void *stream);
 
+/* Sort n candidates by (dm_idx, t, width_idx), as dd_search returns them (host
+ * only).  DD_ERR_ARG for a negative n or a NULL array. */
+DD_API int dd_sort_candidates(dd_candidate *cands, int64_t n);
+
 /* mu and sigma used by the last dd_search on this plan (Section 3; the
  * whole buffer's statistics also when per-row statistics are enabled). */
 DD_API int dd_last_stats(const dd_plan *plan, double *mu, double *sigma);

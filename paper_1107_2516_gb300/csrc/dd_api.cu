@@ -7,6 +7,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <new>
 
 namespace dd {
@@ -96,7 +97,9 @@ static int ensure_cands(dd_plan *p, int64_t cap)
 }
 
 // Sort by (dm_idx, t, width_idx).  Many hits (a strong pulse has thousands): by
-// a 64-bit key, least significant digits first.
+// a 64-bit key, least significant digits first, with 64 bytes of scratch per
+// hit; in place by comparisons where those cannot be had (nothing may be thrown
+// through the C boundary).
 static void sort_candidates(dd_candidate *c, size_t n)
 {
     auto less = [](const dd_candidate &a, const dd_candidate &b) {
@@ -114,21 +117,27 @@ static void sort_candidates(dd_candidate *c, size_t n)
         wi = std::max(wi, (uint64_t)c[i].width_idx);
     }
     const int bt = n ? bits((uint64_t)(t1 - t0)) : 0, bw = bits(wi), all = bits(dm) + bt + bw;
-    if (n < 256 || all > 63) { std::sort(c, c + n, less); return; }
     struct Key { uint64_t key; uint32_t at; };
-    std::vector<Key> a(n), b(n);
+    std::unique_ptr<Key[]> a, b;
+    std::unique_ptr<dd_candidate[]> in;
+    if (n >= 256 && n <= UINT32_MAX && all <= 63) {
+        a.reset(new (std::nothrow) Key[n]);
+        b.reset(new (std::nothrow) Key[n]);
+        in.reset(new (std::nothrow) dd_candidate[n]);
+    }
+    if (!a || !b || !in) { std::sort(c, c + n, less); return; }
     for (size_t i = 0; i < n; ++i)
         a[i] = {(((uint64_t)c[i].dm_idx << bt | (uint64_t)(c[i].t - t0)) << bw) | (uint64_t)c[i].width_idx, (uint32_t)i};
     constexpr int kBits = 11;
     for (int sh = 0; sh < all; sh += kBits) {
         uint32_t at[1 << kBits] = {};
-        for (const Key &k : a) ++at[k.key >> sh & ((1 << kBits) - 1)];
+        for (size_t i = 0; i < n; ++i) ++at[a[i].key >> sh & ((1 << kBits) - 1)];
         uint32_t sum = 0;
         for (uint32_t &v : at) { const uint32_t m = v; v = sum; sum += m; }
-        for (const Key &k : a) b[at[k.key >> sh & ((1 << kBits) - 1)]++] = k;
+        for (size_t i = 0; i < n; ++i) b[at[a[i].key >> sh & ((1 << kBits) - 1)]++] = a[i];
         a.swap(b);
     }
-    const std::vector<dd_candidate> in(c, c + n);
+    std::copy(c, c + n, in.get());
     for (size_t i = 0; i < n; ++i) c[i] = in[a[i].at];
 }
 
@@ -433,6 +442,13 @@ int dd_search(dd_plan *plan, const void *out_dev, dd_candidate *cand_host, int64
     plan->cand_cap = saved_cap;
     if (rc) return rc;
     return search_readback(plan, cand_host, capacity, n_found, s, dev_cap);
+}
+
+int dd_sort_candidates(dd_candidate *cands, int64_t n)
+{
+    if (n < 0 || (n > 0 && !cands)) return set_error(DD_ERR_ARG, "bad candidate array");
+    sort_candidates(cands, (size_t)n);
+    return DD_OK;
 }
 
 int dd_plan_set_search_stats(dd_plan *plan, int32_t per_row)

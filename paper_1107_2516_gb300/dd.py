@@ -31,7 +31,7 @@ EXPORTS = ("dd_plan_create", "dd_plan_destroy", "dd_plan_info", "dd_execute", "d
            "dd_stats_f32_noalloc", "dd_last_error", "dd_version",
            "dd_batch_create", "dd_batch_destroy", "dd_batch_execute", "dd_batch_capture",
            "dd_batch_launch", "dd_batch_results", "dd_batch_autotune", "dd_batch_info", "dd_batch_set_config", "dd_batch_beam_config",
-           "dd_batch_set_launch_mode", "dd_batch_launch_mode", "dd_share_tables", "dd_share_ws_tables", "dd_share_run_tables",
+           "dd_batch_set_launch_mode", "dd_batch_launch_mode", "dd_share_tables", "dd_share_ws_tables", "dd_share_run_tables", "dd_sort_candidates",
            "dd_host_chunk_schedule",
            "dd_server_create", "dd_server_destroy", "dd_server_add_beam", "dd_server_remove_beam",
            "dd_server_submit", "dd_server_poll", "dd_server_candidates", "dd_server_beam_info",
@@ -120,6 +120,7 @@ def load(path: Optional[str] = None):
             "dd_server_candidates": (C.c_int, [vp, i32, i64, vp, i64, P64]),
             "dd_server_beam_info": (C.c_int, [vp, i32, P64, P64, P64, C.POINTER(vp), P64]),
             "dd_server_memory": (C.c_int, [vp, P64, P64]),
+            "dd_sort_candidates": (C.c_int, [vp, i64]),
             "dd_plan_get_launch": (C.c_int, [vp, vp, i64] + [C.POINTER(i32)] * 4),
             "dd_plan_get_tile": (C.c_int, [vp, C.POINTER(i32), C.POINTER(i32), C.POINTER(i32),
                                            C.POINTER(i32)]),
@@ -851,6 +852,12 @@ def dd_channelise(volt_dev, npol: int, nsub: int, nsamp: int, nfft: int, out_dev
 
 
 # ------------------------------------------------------------------ candidate clustering
+
+def dd_sort_candidates(cands: np.ndarray) -> None:
+    """Sorts a CANDIDATE_DTYPE array in place by (dm_idx, t, width_idx), as searches return it."""
+    assert cands.dtype == CANDIDATE_DTYPE and cands.flags.c_contiguous
+    _check(load().dd_sort_candidates(cands.ctypes.data if len(cands) else None, len(cands)))
+
 
 def dd_cluster_candidates(cands: np.ndarray, dm_link: int, t_link: int):
     """Friends-of-friends clusters of a candidate array (CANDIDATE_DTYPE).
