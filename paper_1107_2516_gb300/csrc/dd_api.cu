@@ -75,6 +75,7 @@ static void free_plan(dd_plan *p)
     if (p->d_fin) cudaFree(p->d_fin);
     if (p->d_wsorted) cudaFree(p->d_wsorted);
     if (p->d_cands) cudaFree(p->d_cands);
+    for (dd_candidate *q : p->old_cands) cudaFree(q);
     if (p->h_back) cudaFreeHost(p->h_back);
     if (p->h_cands) cudaFreeHost(p->h_cands);
     if (p->d_rowprm) cudaFree(p->d_rowprm);
@@ -87,7 +88,15 @@ static void free_plan(dd_plan *p)
 static int ensure_cands(dd_plan *p, int64_t cap)
 {
     if (cap <= p->cand_cap) return DD_OK;
-    if (p->d_cands) cudaFree(p->d_cands);
+    // A batch's captured graph writes to the buffer it was captured with, and its
+    // results are read from there: that one stays.  The next is at least twice
+    // the size, so that what stays is less than what is used.
+    if (p->in_graph) {
+        p->old_cands.push_back(p->d_cands);
+        cap = std::max(cap, 2 * p->cand_cap);
+    } else if (p->d_cands) {
+        cudaFree(p->d_cands);
+    }
     p->d_cands = nullptr;
     p->cand_cap = 0;
     cudaError_t e = cudaMalloc(&p->d_cands, (size_t)cap * sizeof(dd_candidate));
@@ -142,17 +151,17 @@ static void sort_candidates(dd_candidate *c, size_t n)
 }
 
 // Synchronise `s`, read the search results of the plan's last search_launch
-// (dev_cap = the candidate capacity that launch used) and sort them.  The
+// (dev_cands, dev_cap = the candidate buffer that launch used) and sort them.  The
 // first candidates come with the count and the status: one wait for the usual
 // search instead of three (execute and search of 64 trials x 6600 samples 97 ->
 // 77 us; 8 beams' results with 23 000 hits, sort included, 1.2 -> 0.6 ms).
 int search_readback(dd_plan *plan, dd_candidate *cand_host, int64_t capacity, int64_t *n_found,
-                    cudaStream_t s, int64_t dev_cap)
+                    cudaStream_t s, const dd_candidate *dev_cands, int64_t dev_cap)
 {
     const int64_t most = std::min(dev_cap, capacity), pre = std::min<int64_t>(most, kBackCands);
     cudaError_t e = cudaMemcpyAsync(plan->h_back, plan->d_back, sizeof(SearchBack), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess && pre > 0)
-        e = cudaMemcpyAsync(plan->h_cands, plan->d_cands, (size_t)pre * sizeof(dd_candidate), cudaMemcpyDeviceToHost, s);
+        e = cudaMemcpyAsync(plan->h_cands, dev_cands, (size_t)pre * sizeof(dd_candidate), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess && plan->row_stats && plan->d_rowprm)
         e = cudaMemcpyAsync(plan->h_rowprm, plan->d_rowprm, (size_t)plan->ndm * sizeof(RowParams),
                             cudaMemcpyDeviceToHost, s);
@@ -168,7 +177,7 @@ int search_readback(dd_plan *plan, dd_candidate *cand_host, int64_t capacity, in
     plan->last_sigma = plan->h_back->prm.sigma;
     if (n > 0) memcpy(cand_host, plan->h_cands, (size_t)std::min(n, pre) * sizeof(dd_candidate));
     if (n > pre) {
-        e = cudaMemcpyAsync(cand_host + pre, plan->d_cands + pre, (size_t)(n - pre) * sizeof(dd_candidate),
+        e = cudaMemcpyAsync(cand_host + pre, dev_cands + pre, (size_t)(n - pre) * sizeof(dd_candidate),
                             cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return cuda_fail(e, "candidate readback");
@@ -441,7 +450,7 @@ int dd_search(dd_plan *plan, const void *out_dev, dd_candidate *cand_host, int64
     const int64_t dev_cap = plan->cand_cap;
     plan->cand_cap = saved_cap;
     if (rc) return rc;
-    return search_readback(plan, cand_host, capacity, n_found, s, dev_cap);
+    return search_readback(plan, cand_host, capacity, n_found, s, plan->d_cands, dev_cap);
 }
 
 int dd_sort_candidates(dd_candidate *cands, int64_t n)

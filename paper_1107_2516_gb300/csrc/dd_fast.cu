@@ -1262,6 +1262,8 @@ struct dd_batch {
     int grid = 0;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
+    std::vector<std::pair<dd_candidate *, int64_t>> graph_cands;   // the plans' candidate buffers at capture
+    bool replayed = false;                 // the last run was the graph's
 };
 
 namespace dd {
@@ -1684,6 +1686,7 @@ int dd_batch_destroy(dd_batch *B)
 int dd_batch_execute(dd_batch *B, const void *const *ins, const int64_t *pitches, void *const *outs, void *stream)
 {
     if (!B || !ins || !pitches || !outs) return set_error(DD_ERR_ARG, "NULL argument");
+    B->replayed = false;
     return batch_enqueue(B, ins, pitches, outs, (cudaStream_t)stream);
 }
 
@@ -1706,6 +1709,11 @@ int dd_batch_capture(dd_batch *B, const void *const *ins, const int64_t *pitches
     B->graph = g;
     e = cudaGraphInstantiate(&B->exec, g, 0);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate");
+    B->graph_cands.clear();
+    for (dd_plan *p : B->plans) {
+        B->graph_cands.emplace_back(p->d_cands, p->cand_cap);
+        p->in_graph = true;
+    }
     return DD_OK;
 }
 
@@ -1714,6 +1722,7 @@ int dd_batch_launch(dd_batch *B, void *stream)
     if (!B || !B->exec) return set_error(DD_ERR_ARG, "no captured graph");
     cudaError_t e = cudaGraphLaunch(B->exec, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGraphLaunch");
+    B->replayed = true;
     return DD_OK;
 }
 
@@ -1731,7 +1740,8 @@ int dd_batch_results(dd_batch *B, int32_t beam, dd_candidate *cand_host, int64_t
         if (h) return set_error(h, "batch kernel gave up waiting for its input copies");
     }
     dd_plan *p = B->plans[beam];
-    return search_readback(p, cand_host, capacity, n_found, s, p->cand_cap);
+    const auto cands = B->replayed ? B->graph_cands[beam] : std::make_pair(p->d_cands, p->cand_cap);
+    return search_readback(p, cand_host, capacity, n_found, s, cands.first, cands.second);
 }
 
 int dd_batch_autotune(dd_batch *B, const void *const *ins, const int64_t *pitches, void *const *outs, void *stream)

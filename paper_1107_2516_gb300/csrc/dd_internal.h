@@ -100,6 +100,8 @@ struct dd_plan {
     dd::FinScratch *d_fin = nullptr;
     int32_t *d_wsorted = nullptr;          // widths sorted ascending: [nw] widths, [nw] indices
     dd_candidate *d_cands = nullptr;
+    bool in_graph = false;                 // a batch's captured graph has held d_cands
+    std::vector<dd_candidate *> old_cands; // outgrown since then: the graph writes there
     int64_t cand_cap = 0;
     unsigned long long *d_count = nullptr; // in d_back
     dd_candidate *h_cands = nullptr;       // pinned [kBackCands]
@@ -146,7 +148,7 @@ int ensure_partials_public(dd_plan *p, int64_t n);
 int boundary_search_launch(dd_plan *p, const void *tail, const void *out, int L, cudaStream_t s);
 long long max_delay(int nchans, double fch1, double foff, double tsamp_s, const double *dm_list, int ndm);
 int search_readback(dd_plan *plan, dd_candidate *cand_host, int64_t capacity, int64_t *n_found,
-                    cudaStream_t s, int64_t dev_cap);
+                    cudaStream_t s, const dd_candidate *dev_cands, int64_t dev_cap);
 cudaError_t allow_max_dynamic_smem(const void *fn, size_t optin);
 
 // dd_fast.cu

@@ -154,7 +154,7 @@ static void process(dd_server *S, ServerBeam *b, const Pending &pc, cudaStream_t
                 int64_t nb = 0;
                 rc2 = boundary_search_launch(b->plan, b->tail, b->out, b->L, s);
                 if (rc2 == DD_OK)
-                    rc2 = search_readback(b->plan, bnd.data(), S->cand_cap, &nb, s, b->plan->cand_cap);
+                    rc2 = search_readback(b->plan, bnd.data(), S->cand_cap, &nb, s, b->plan->d_cands, b->plan->cand_cap);
                 if (rc2 == DD_OK || rc2 == DD_ERR_OVERFLOW) {
                     const dd_plan *p = b->plan;
                     for (int64_t i = 0; i < std::min(nb, S->cand_cap); ++i) {

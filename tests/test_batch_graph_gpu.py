@@ -57,3 +57,32 @@ def test_replay_after_the_plans_ran_alone(dtype):
     batch.close()
     for p in plans:
         p.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "u8"])
+def test_replay_after_a_larger_search(dtype):
+    # a search with room for more candidates than the graph was captured with
+    plans, ins, outs = beams(dtype)
+    s = torch.cuda.Stream()
+    batch = dd.Batch(plans)
+    batch.capture(ins, [9216] * 2, outs, s)
+    first = results(batch, plans, s)
+    other = []
+    for p, x, o in zip(plans, ins, outs):
+        out = torch.zeros_like(o)
+        p.execute(x, 9216, out)
+        out.zero_()                                # what the plan's own search finds last is not the batch's
+        other.append(p.search(out, capacity=1 << 20)[1])
+    torch.cuda.synchronize()
+    fill = [torch.full((1 << k,), 255, dtype=torch.uint8, device="cuda") for k in range(10, 23)]
+    second = results(batch, plans, s)
+    assert same(first, second) and all(n != m for (_, n, _), m in zip(first, other))
+    assert all(bool((f == 255).all()) for f in fill)
+    # run directly, the batch takes the plans' buffers of now
+    batch.execute(ins, [9216] * 2, outs)
+    for i, p in enumerate(plans):
+        c, n = batch.results(i)
+        assert n == first[i][1] and np.array_equal(c, first[i][0])
+    batch.close()
+    for p in plans:
+        p.close()
