@@ -261,8 +261,12 @@ DD_API int dd_plan_get_tile(const dd_plan *plan, int32_t *config, int32_t *raste
  * different channel counts, lengths, DM grids and input types) in ONE
  * persistent launch that pulls (beam, DM block, time tile) work items from a
  * device queue ordered heaviest first, followed by each beam's Section 3
- * search.  Each beam's output and candidates are those its plan alone would
- * produce (the same arithmetic in the same order).
+ * search.  Each beam's output and candidates are those its plan alone produces
+ * in the configuration that dd_batch_beam_config reports (dd_plan_set_tile): the
+ * same arithmetic in the same order, the same bits.  DD_U8 sums are the same bits in
+ * every configuration.  A floating-point plan left to itself may sum in another
+ * order (configuration 12 may sum 8 channels before it adds them, the persistent
+ * grid 4 or 1): the same sums to rounding.
  * ------------------------------------------------------------------- */
 
 /* Group `nplans` plans (not owned; they must outlive the batch and live on
