@@ -133,7 +133,10 @@ DD_API int dd_plan_info(const dd_plan *plan, int64_t *maxshift, int64_t *nsamp_o
  * elements per channel row (in_pitch >= nsamp_in).  out_dev: device pointer
  * to D*nsamp_out float32 (int32 for DD_U8).  stream: a cudaStream_t (NULL =
  * legacy default stream).  Asynchronous: returns after the launches are
- * queued.  The input buffers must not alias. */
+ * queued.  The input buffers must not alias.  Rows are copied in the whole
+ * 16-byte units that hold their samples: up to 15 bytes before a row's first
+ * sample and behind its last one are read (never beyond the unit, so never
+ * beyond a page) and not used; they may change meanwhile. */
 DD_API int dd_execute(dd_plan *plan, const void *in_dev, int64_t in_pitch, void *out_dev,
                void *stream);
 
