@@ -106,6 +106,16 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, int *e
     return true;
 }
 
+// The rest of an item for a warp whose wait for stage s of n gave up: it issues no
+// copies and follows no offsets or records that did not land, lets the copies
+// in flight (stages s to s + ring - 1, counted from g0) land, and meets the
+// others at their barriers, one per stage.  Their waits give up too.
+__device__ __forceinline__ void sit_out(uint64_t *bar, uint32_t g0, int s, int n, int ring, int *err)
+{
+    for (int u = s; u < min(s + ring, n); ++u) mbar_wait(&bar[(g0 + u) % ring], ((g0 + u) / ring) & 1u, err);
+    for (; s < n; ++s) __syncthreads();
+}
+
 __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
 {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"

@@ -247,7 +247,8 @@ __device__ __forceinline__ bool lane_tile(const LaneLaunch &a, int blk, int64_t 
         if (s + kStages - 1 < nst) issue(s + kStages - 1);
         const uint32_t g = g0 + s;
         const int buf = (int)(g % kStages);
-        if (ok) ok = mbar_wait(&bar[buf], (g / kStages) & 1u, a.err);
+        ok = __all_sync(0xffffffffu, mbar_wait(&bar[buf], (g / kStages) & 1u, a.err));
+        if (!ok) { sit_out(bar, g0, s, nst, kStages, a.err); break; }
         const int cn = idle ? 0 : min(ch, nchans - s * ch);
         const Tin *srow = rows + (size_t)buf * stage_elems + lane;
         const int32_t *so = soffs + (size_t)buf * ch * kDmBlk + warp * DR;

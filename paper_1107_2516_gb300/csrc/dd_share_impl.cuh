@@ -443,7 +443,8 @@ __device__ __forceinline__ bool share_tile(const ShareLaunch &a, int blk, int64_
             if (s + NS < nsub) load_rb(s + NS);
         }
         const int buf = (int)((g0 + s) % NS);
-        if (ok) ok = mbar_wait(&bar[buf], (uint32_t)(((g0 + s) / NS) & 1), a.err);
+        ok = __all_sync(0xffffffffu, mbar_wait(&bar[buf], (uint32_t)(((g0 + s) / NS) & 1), a.err));
+        if (!ok) { sit_out(bar, g0, s, nsub, NS, a.err); break; }
         const int32_t *rec = srec + (size_t)buf * R::kLen;
         const Tin *srow = rows + (size_t)buf * stage_elems;
         float *Pb = P + (size_t)(s & 1) * a.pmax;

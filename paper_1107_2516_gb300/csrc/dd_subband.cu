@@ -138,7 +138,8 @@ __global__ void __launch_bounds__(NW * 32, 3) sub_kernel(SubLaunch a)
     for (int s = 0; s < nst; ++s) {
         if (s + kStages - 1 < nst) issue(s + kStages - 1);
         const int buf = s % kStages;
-        if (ok) ok = mbar_wait(&bar[buf], (uint32_t)((s / kStages) & 1), a.err);
+        ok = __all_sync(0xffffffffu, mbar_wait(&bar[buf], (uint32_t)((s / kStages) & 1), a.err));
+        if (!ok) { sit_out(bar, 0, s, nst, kStages, a.err); break; }
         const int cn = idle ? 0 : min(ch, nchans - s * ch);
         const Tin *srow = rows + (size_t)buf * stage_elems + lane;
         const int32_t *so = soffs + (size_t)buf * ch * kDmBlk + warp * DR;
