@@ -179,8 +179,8 @@ DD_API int dd_last_row_stats(const dd_plan *plan, double *mu_rows, double *sigma
  * and dd_search, and returns the candidates as dd_search does.  With
  * kernels 3 and 5 the copy goes in 8 column chunks on a stream of the plan,
  * and the output tiles each chunk completes are de-dispersed while the next
- * chunk is in flight (same results as the unsplit call; a launch of few
- * blocks is not split).  The plan allocates
+ * chunk is in flight (same results as the unsplit call; a launch of no more
+ * blocks than SMs is not split).  The plan allocates
  * its device staging for `in` and `out` on the first call and keeps it until
  * dd_plan_destroy.  Synchronises `stream`. */
 DD_API int dd_process_host(dd_plan *plan, const void *in_host, int64_t in_pitch,
