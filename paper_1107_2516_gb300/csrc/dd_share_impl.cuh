@@ -197,7 +197,7 @@ __device__ __forceinline__ void share_stage1(const int32_t *rec, const Tin *srow
 // Per quad and lane 2 CS + 4 shared words for four sums, against 4 (CS + 1)
 // with one byte load (and a conversion to float) per term; stage 2 reads half
 // the words.  Bound by instructions, no longer by shared memory (ncu: issue
-// 71%, shared-memory wavefronts 60% of their peaks).  LOFAR-like beam of 2^18
+// 75%, shared-memory wavefronts 65% of their peaks).  LOFAR-like beam of 2^18
 // uint8 samples, 2000 trials: 30.0 -> 20.2 ms; 4096 channels x 65536 samples,
 // 1500 trials: 24.7 -> 13.5 ms.  Exact step sizes for the rows that are left,
 // and the high half added with one dp2a instead of a shift and an add, are
