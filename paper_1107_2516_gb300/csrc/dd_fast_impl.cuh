@@ -108,11 +108,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, int *e
 
 // The rest of an item for a warp whose wait for stage s of n gave up: it issues no
 // copies and follows no offsets or records that did not land, lets the copies
-// in flight (stages s to s + ring - 1, counted from g0) land, and meets the
-// others at their barriers, one per stage.  Their waits give up too.
+// in flight (stages s to s + ring - 1, counted from g0) land for up to 0.2 s each,
+// and meets the others at their barriers, one per stage.  Their waits give up too.
 __device__ __forceinline__ void sit_out(uint64_t *bar, uint32_t g0, int s, int n, int ring, int *err)
 {
-    for (int u = s; u < min(s + ring, n); ++u) mbar_wait(&bar[(g0 + u) % ring], ((g0 + u) / ring) & 1u, err);
+    for (int u = s; u < min(s + ring, n); ++u)
+        mbar_wait(&bar[(g0 + u) % ring], ((g0 + u) / ring) & 1u, err, kWaitLimitNs / 10);
     for (; s < n; ++s) __syncthreads();
 }
 
