@@ -542,7 +542,7 @@ static int share_ws_stages(const ShareTables &T, int cs, int rs, size_t eb, size
 // with 4 and 2.68 ms with 8; 4096 channels over 200 MHz, uint8 (9.4 patterns)
 // 14.1 ms with 4 and 15.2 ms with 8.  Over 288 launches (64 to 4096 channels at 150
 // to 1500 MHz, DM steps 0.01 to 1, each type) 8 is taken in 153 and is the faster one
-// in each, by 1% to 44%.
+// in each, 1.01 to 2.0 times as fast.
 // T.ok is false where subbands of 4 have too many patterns or do not fit.
 static int share_ws_choose(const int32_t *d, int D, int C, double foff, dd_dtype dtype, size_t optin, ShareTables &T)
 {
